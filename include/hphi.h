@@ -165,7 +165,9 @@ HPHI_API int64_t hphi_ham_dim(const hphi_ham *ham);
  *   HPHI_TUNE_SPLIT       thread blocks that share one row block (1..8),
  *                         fewer row blocks in flight for the same occupancy
  *   HPHI_TUNE_L2_HINTS    1 = L2 eviction-priority hints on gathers/streams
- *   HPHI_TUNE_VARIANT     -1 = automatic (default); spin models: 1 = neighbour
+ *   HPHI_TUNE_VARIANT     -1 = automatic (default; one column of an S^z sector
+ *                         takes the segment kernel, which has no number of
+ *                         its own); spin models: 1 = neighbour
  *                         ranks computed on the fly from Lin's ja table, 0 =
  *                         precomputed neighbour lists (also enables the
  *                         one-thread-per-row kernel for Hubbard), 2 = staged:

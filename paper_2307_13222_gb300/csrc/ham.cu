@@ -144,6 +144,8 @@ void free_ham(hphi_ham *h) {
     cudaFree(h->dterms_d);
     cudaFree(h->rowstate);
     cudaFree(h->seg_so);
+    cudaFree(h->warp_tab);
+    delete h->warp;
     for (int p = 0; p < 2; p++) {
         cudaFree(h->tile_tab[p]);
         cudaFree(h->tile_diag[p]);
@@ -313,7 +315,7 @@ int build_spin(hphi_ctx *ctx, hphi_ham *H, const hphi_term *terms, int n_terms) 
     cudaFree(d_lb);
     if (e != cudaSuccess) return cuda_err(ctx, e, "k_spin_tables");
     if (sector && nlo <= 16 && ll.size() <= 128 && (st = build_bond_lists(ctx, H, ll, lowbits))) return st;
-    if (sector && (st = build_seg_tables(ctx, H))) return st;
+    if (sector && ((st = build_seg_tables(ctx, H)) || (st = build_warp_tables(ctx, H)))) return st;
     return HPHI_OK;
 }
 

@@ -108,6 +108,25 @@ struct SegArgs {
     const uint16_t *so;  // [(N_lo + 1) << n1]
 };
 
+// Segment kernel (hv_warp.cu): the lowest s bits form the segments, the other
+// n1 bits of the low half and the high half pick one.
+constexpr int kWarpSegMax = 10;  // most segment bits
+struct WarpClass {   // segments of one popcount: rows, rows per lane, offsets of their table parts
+    uint32_t len;
+    int nc, row0, tab;
+};
+struct WarpArgs {
+    int s, n1, nlo, n, rot;
+    int nu, nx, nm, ni;           // uniform, mixed, mixed diagonal, inner bonds
+    int nrow, tab_stride, ntab;   // padded rows of all classes, bytes of a table, tables of the mixed bonds
+    double scale64, scale32;      // fixed point to value
+    int moff[kWarpSegMax + 1];    // mixed diagonal entries of each segment bit
+    uint8_t order[64];            // segments of a row block, long ones first
+    WarpClass cls[kWarpSegMax + 1];
+    int jl, jw, jhi;              // Lin's jb in two parts: low and high bits of h, 2^jw
+    const unsigned char *img32, *img64;  // device: the tables' images (hv_warp.cu, WarpLayout)
+};
+
 // Lin tables of one species (spin string, or up / down fermion string).
 struct Species {
     int N = 0, n = 0, nlo = 0, nhi = 0;
@@ -199,6 +218,10 @@ struct hphi_ham {
     // arguments (null when not available) and its device table
     hphi::SegArgs *seg = nullptr;
     uint16_t *seg_so = nullptr;
+    // segment kernel (spin S^z sector): host copy of its arguments (null when not
+    // available) and its device tables
+    hphi::WarpArgs *warp = nullptr;
+    unsigned char *warp_tab = nullptr;
     // tiled block kernel (full space, 32 columns), per precision [0: FP32, 1: FP64]
     // (the tiles follow the row size): built on first use
     hphi::TileArgs *tile[2] = {nullptr, nullptr};
@@ -324,6 +347,8 @@ int lowest_ritz_warm(int m, const double *alpha, const double *beta2, double *wa
 
 // ---- high-high pass table (hv_seg.cu) ------------------------------------------------
 int build_seg_tables(hphi_ctx *ctx, hphi_ham *H);
+// ---- segment kernel tables (hv_warp.cu) ----------------------------------------------
+int build_warp_tables(hphi_ctx *ctx, hphi_ham *H);
 // ---- tiled block kernel tables (hv_tile.cu) ------------------------------------------
 int build_tile_tables(hphi_ctx *ctx, hphi_ham *H, int prec);
 

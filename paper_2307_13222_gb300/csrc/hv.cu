@@ -311,7 +311,15 @@ int launch_typed(hphi_ctx *ctx, const hphi_ham *ham, HvLaunch &L) {
         const bool hub_phased = (ham->tune_variant == 3 || ham->tune_variant < 0) && ham->model == HPHI_HUBBARD &&
                                 ham->ph_ent && one_col &&
                                 (double)ham->basis->sp[1].dim * 2.0 * sizeof(T) <= 200.0 * 1024.0;
-        const bool staged = spin_staged || hub_phased || seg;
+        // the segment kernel: spin sector, one column, automatic where its tables exist.  It
+        // issues its mixed-bond FMAs for every row and the bond-major kernel only where they
+        // apply, so in FP64, where the FP64 pipe bounds both, the latter stays where its lists
+        // are longest (row blocks of 16 low bits: 4x8 56.9 against 62.3 ms; 15 bits: 6x5 15.5
+        // against 15.2).  FP32 problems below 2^14 rows keep the bond-major kernel too: both
+        // are one wave of latency there (16 sites: 10 us).
+        const bool warp = ham->tune_variant < 0 && ham->warp && one_col &&
+                          (std::is_same<T, double>::value ? ham->nlo < 16 : ham->D >= 16384);
+        const bool staged = spin_staged || hub_phased || seg || warp;
         // spin models: the on-the-fly-rank kernel for unit / pair / 32-wide rows
         int fG = 0, fcpl = 0;
         // variant -1 (automatic): on-the-fly ranks for 32-wide rows, lists for unit / pair rows
@@ -412,7 +420,8 @@ int launch_typed(hphi_ctx *ctx, const hphi_ham *ham, HvLaunch &L) {
             // the staged kernel on the 6x5 and 4x8 sectors, FP32 and FP64)
             const bool phased = hub_phased || ham->tune_variant == 3 ||
                                 (ham->tune_variant < 0 && ham->ph_ent && ham->host.n_ll <= 128);
-            st = seg ? launch_seg<T>(ctx, ham, a, red_mode, &grid)
+            st = seg    ? launch_seg<T>(ctx, ham, a, red_mode, &grid)
+                 : warp ? launch_warp<T>(ctx, ham, a, red_mode, &grid)
                      : phased ? launch_phased<T>(ctx, ham, a, red_mode, &grid)
                               : launch_staged<T>(ctx, ham, a, red_mode, &grid);
         } else if (fG) {

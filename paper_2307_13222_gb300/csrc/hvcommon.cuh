@@ -113,6 +113,7 @@ inline HvTables make_tables(const hphi_ham *ham, int real_dtype) {
     P.ngroups = ham->host.ngroups;
     P.n = ham->host.n;
     P.nh = ham->nh;
+    P.rows = ham->D;
     P.L = ham->L;
     P.ddn = ham->host.ddn;
     P.jb = b->sp[0].jb;
@@ -224,6 +225,9 @@ uint32_t staged_block_len(const hphi_ham *ham);
 // tiled two-pass block kernel (hv_tile.cu): full space, 32 columns (FP32 or FP64)
 template <typename T>
 int launch_tile(hphi_ctx *ctx, const hphi_ham *ham, HvArgs<T> &a, int red_mode, int *grid);
+// segment kernel (hv_warp.cu): spin sector, one column
+template <typename T>
+int launch_warp(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int red_mode, int *grid);
 // high-high pass plus the bond-major kernel (hv_seg.cu): spin sector, one column
 template <typename T>
 int launch_seg(hphi_ctx *ctx, const hphi_ham *ham, HvArgs<T> &a, int red_mode, int *grid);

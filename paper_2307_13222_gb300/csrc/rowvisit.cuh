@@ -21,6 +21,7 @@ struct HvTables {
     int model;
     int nlo, ngroups, n;
     int64_t nh, L, ddn;
+    int64_t rows;            // dimension
     // spin species tables
     const uint64_t *jb;
     const uint32_t *loff;
