@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "hphi_internal.cuh"
+#include "reduce.cuh"
 
 namespace hphi {
 
@@ -225,62 +226,69 @@ int lowest_ritz(int m, const double *alpha, const double *beta2, double *theta, 
 
 namespace {
 
-enum LzMode { LZ_INIT = 0, LZ_PREP_A = 1, LZ_ALPHA = 2, LZ_BETA = 3 };
+// Scalar bookkeeping of the device-side recurrence: one thread block sums the
+// partials of the launch before it (grid of them, `stride` apart), thread 0
+// derives the next coefficients.  A step is four launches: H*x, LZ_ALPHA, the
+// combination, LZ_BETA.
+enum LzMode { LZ_INIT = 0, LZ_ALPHA = 1, LZ_BETA = 2 };
 
-// one thread: scalar bookkeeping of the device-side recurrence
-__global__ void k_lz(int mode, int k, const double *red, double *alpha, double *beta2, double *coefA, double *coefB,
-                     int *flag) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void __launch_bounds__(kSumThreads)
+    k_lz(int mode, int k, const double *part, int grid, int stride, double *alpha, double *beta2, double *coefA,
+         double *coefB, int *flag) {
+    const double red = block_sum_strided(part, grid, stride);
+    if (threadIdx.x != 0) return;
     // *flag records the first step (k + 1) whose scalars were not finite; -1
     // marks a start vector of zero norm
     if (mode == LZ_INIT) {
-        beta2[0] = red[0];
-        if (!(red[0] > 0.0) || !isfinite(red[0])) *flag = -1;
-    } else if (mode == LZ_PREP_A) {
-        double bk = sqrt(beta2[k]);
-        coefA[0] = 1.0 / bk;
-        coefA[1] = k > 0 ? -bk / sqrt(beta2[k - 1]) : 0.0;
+        beta2[0] = red;
+        if (!(red > 0.0) || !isfinite(red)) *flag = -1;
+        coefA[0] = 1.0 / sqrt(red);
+        coefA[1] = 0.0;
     } else if (mode == LZ_ALPHA) {
-        double bk = sqrt(beta2[k]);
-        double a = red[0] / bk;
+        const double bk = sqrt(beta2[k]), a = red / bk;
         alpha[k] = a;
         coefB[0] = -a / bk;  // coefficient of w_k
         coefB[1] = 0.0;
         coefB[2] = 1.0;      // coefficient of u
         if (!isfinite(a) && *flag == 0) *flag = k + 1;
     } else {
-        beta2[k + 1] = red[0];
-        if ((!(red[0] >= 0.0) || !isfinite(red[0])) && *flag == 0) *flag = k + 1;
+        beta2[k + 1] = red;
+        if ((!(red >= 0.0) || !isfinite(red)) && *flag == 0) *flag = k + 1;
+        const double bn = sqrt(red);  // the next step's H*x coefficients
+        coefA[0] = 1.0 / bn;
+        coefA[1] = -bn / sqrt(beta2[k]);
     }
 }
 
-// scalar bookkeeping of the reorthogonalising recurrence (normalised vectors)
-enum RzMode { RZ_INIT = 0, RZ_PREP = 1, RZ_ALPHA = 2, RZ_BETA = 3 };
+// The same for the reorthogonalising recurrence (normalised vectors).
+enum RzMode { RZ_INIT = 0, RZ_ALPHA = 1, RZ_BETA = 2 };
 
-__global__ void k_rz(int mode, int k, const double *red, double *alpha, double *beta2, double *coef, int *flag) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    if (mode == RZ_INIT) {
-        beta2[0] = red[0];
-        if (!(red[0] > 0.0) || !isfinite(red[0])) *flag = -1;
-        coef[0] = 1.0 / sqrt(red[0]);  // scale of v_0
-        coef[1] = 0.0;
-        coef[2] = 0.0;
-    } else if (mode == RZ_PREP) {
-        coef[0] = 1.0;                               // alpha of H*x
-        coef[1] = k > 0 ? -sqrt(beta2[k]) : 0.0;     // gamma: -beta_k v_{k-1}
-    } else if (mode == RZ_ALPHA) {
-        alpha[k] = red[0];
-        coef[0] = -red[0];  // u -= alpha_k v_k
-        coef[1] = 0.0;
-        coef[2] = 1.0;
-        if (!isfinite(red[0]) && *flag == 0) *flag = k + 1;
-    } else {
-        beta2[k + 1] = red[0];
-        coef[0] = 1.0 / sqrt(red[0]);  // v_{k+1} = u / beta_{k+1}
-        coef[1] = 0.0;
-        coef[2] = 0.0;
-        if ((!(red[0] >= 0.0) || !isfinite(red[0])) && *flag == 0) *flag = k + 1;
+__global__ void __launch_bounds__(kSumThreads)
+    k_rz(int mode, int k, const double *part, int grid, int stride, double *alpha, double *beta2, double *coefA,
+         double *coefB, int *flag) {
+    const double red = block_sum_strided(part, grid, stride);
+    if (threadIdx.x != 0) return;
+    if (mode == RZ_ALPHA) {
+        alpha[k] = red;
+        coefB[0] = -red;  // u -= alpha_k v_k
+        coefB[1] = 0.0;
+        coefB[2] = 1.0;
+        if (!isfinite(red) && *flag == 0) *flag = k + 1;
+        return;
     }
+    const double b = sqrt(red);
+    if (mode == RZ_INIT) {
+        beta2[0] = red;
+        if (!(red > 0.0) || !isfinite(red)) *flag = -1;
+    } else {
+        beta2[k + 1] = red;
+        if ((!(red >= 0.0) || !isfinite(red)) && *flag == 0) *flag = k + 1;
+    }
+    coefB[0] = 1.0 / b;  // v_{k+1} = u / beta_{k+1}
+    coefB[1] = 0.0;
+    coefB[2] = 0.0;
+    coefA[0] = 1.0;                            // the next H*x: H v - beta v_prev
+    coefA[1] = mode == RZ_INIT ? 0.0 : -b;
 }
 
 }  // namespace
@@ -386,11 +394,13 @@ static int lanczos_reorth(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lanczos
     if ((st = ensure_partials(ctx, np))) return st;
     char *Vb = nullptr;
     double *sc = nullptr;
-    cudaError_t e = cudaMalloc((void **)&Vb, vb * ((size_t)M + 1));
+    const int64_t ldv = (D + 3) & ~(int64_t)3;  // every vector on a 16-byte boundary
+    const size_t vs = (size_t)ldv * es;
+    cudaError_t e = cudaMalloc((void **)&Vb, vs * ((size_t)M + 1));
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_err(ctx, HPHI_E_NOMEM, "reorthogonalisation needs %zu bytes for %d Krylov vectors",
-                       vb * ((size_t)M + 1), M + 1);
+                       vs * ((size_t)M + 1), M + 1);
     }
     e = cudaMalloc((void **)&sc, sizeof(double) * (4 * (size_t)M + 16));
     if (e != cudaSuccess) {
@@ -400,7 +410,7 @@ static int lanczos_reorth(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lanczos
     }
     double *alpha_d = sc, *beta2_d = sc + M + 1, *cbuf = sc + 2 * (size_t)M + 4;  // cbuf: M + 1 entries
     double *coefA = ctx->dscal + 3000, *coefB = ctx->dscal + 3008, *red = ctx->dscal + 3016;
-    auto V = [&](int j) -> void * { return Vb + (size_t)j * vb; };
+    auto V = [&](int j) -> void * { return Vb + (size_t)j * vs; };
     auto fail = [&](int code) {
         cudaStreamSynchronize(ctx->stream);
         cudaFree(Vb);
@@ -411,7 +421,7 @@ static int lanczos_reorth(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lanczos
     std::vector<double> alpha_h(M + 1, 0.0), beta2_h(M + 2, 0.0), y;
     int steps = 0, conv = 0, brk = 0;
     double theta = 0.0, resid_est = -1.0, warm = std::nan("");
-    auto lincomb = [&](const void *x, const void *yv, void *out, const double *cdev, int red_oo) -> int {
+    auto lincomb = [&](const void *x, const void *yv, void *out, const double *cdev) -> int {
         LinComb B{};
         B.real_dtype = dt;
         B.n = D;
@@ -423,19 +433,16 @@ static int lanczos_reorth(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lanczos
         B.out = out;
         B.ldo = 1;
         B.coef_dev = cdev;
-        B.red_oo = red_oo;
+        B.red_oo = 0;
         B.partials = ctx->partials;
-        int s2 = launch_lincomb(ctx, B);
-        if (!s2 && red_oo) s2 = reduce_partials(ctx, ctx->partials, B.grid, 1, red);
-        return s2;
+        return launch_lincomb(ctx, B);
     };
     HPHI_CUDA(ctx, cudaMemsetAsync(ctx->dflag, 0, sizeof(int), ctx->stream));
     if ((st = launch_copy(ctx, dt, D, 1, v0, 1, V(0), 1))) return fail(st);
     if ((st = launch_dot(ctx, dt, 0, D, 1, V(0), 1, V(0), 1, red))) return fail(st);
-    k_rz<<<1, 32, 0, ctx->stream>>>(RZ_INIT, 0, red, alpha_d, beta2_d, coefB, ctx->dflag);
-    if ((st = lincomb(V(0), nullptr, V(0), coefB, 0))) return fail(st);
+    k_rz<<<1, kSumThreads, 0, ctx->stream>>>(RZ_INIT, 0, red, 1, 1, alpha_d, beta2_d, coefA, coefB, ctx->dflag);
+    if ((st = lincomb(V(0), nullptr, V(0), coefB))) return fail(st);
     for (int k = 0; k < M; k++) {
-        k_rz<<<1, 32, 0, ctx->stream>>>(RZ_PREP, k, red, alpha_d, beta2_d, coefA, ctx->dflag);
         HvLaunch A{};
         A.dtype_real = dt;
         A.ncol = 1;
@@ -448,17 +455,19 @@ static int lanczos_reorth(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lanczos
         A.coef_dev = coefA;
         A.red[0] = R_XO;
         A.partials = ctx->partials;
-        if ((st = launch_hv(ctx, ham, A)) || (st = reduce_hv(ctx, A, red))) return fail(st);
-        k_rz<<<1, 32, 0, ctx->stream>>>(RZ_ALPHA, k, red, alpha_d, beta2_d, coefB, ctx->dflag);
-        if ((st = lincomb(V(k), u, u, coefB, 0))) return fail(st);
+        if ((st = launch_hv(ctx, ham, A))) return fail(st);
+        k_rz<<<1, kSumThreads, 0, ctx->stream>>>(RZ_ALPHA, k, A.partials, A.sgrid[0], 3, alpha_d, beta2_d, coefA, coefB,
+                                                 ctx->dflag);
+        if ((st = lincomb(V(k), u, u, coefB))) return fail(st);
+        int ng = 0;
         for (int pass = 0; pass < 2; pass++) {
-            if ((st = launch_mdot(ctx, dt, D, k + 1, Vb, u, cbuf)) ||
-                (st = launch_maxpy(ctx, dt, D, k + 1, Vb, cbuf, u)))
+            if ((st = launch_mdot(ctx, dt, D, ldv, k + 1, Vb, u, cbuf)) ||
+                (st = launch_maxpy(ctx, dt, D, ldv, k + 1, Vb, cbuf, u, pass == 1 ? &ng : nullptr)))
                 return fail(st);
         }
-        if ((st = launch_dot(ctx, dt, 0, D, 1, u, 1, u, 1, red))) return fail(st);
-        k_rz<<<1, 32, 0, ctx->stream>>>(RZ_BETA, k, red, alpha_d, beta2_d, coefB, ctx->dflag);
-        if ((st = lincomb(u, nullptr, V(k + 1), coefB, 0))) return fail(st);
+        k_rz<<<1, kSumThreads, 0, ctx->stream>>>(RZ_BETA, k, ctx->partials, ng, 1, alpha_d, beta2_d, coefA, coefB,
+                                                 ctx->dflag);
+        if ((st = lincomb(u, nullptr, V(k + 1), coefB))) return fail(st);
         HPHI_CUDA(ctx, cudaGetLastError());
         steps = k + 1;
         if ((k + 1) % check == 0 || k + 1 == M) {
@@ -518,8 +527,10 @@ static int lanczos_reorth(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lanczos
         std::vector<double> ny(m);
         for (int j = 0; j < m; j++) ny[j] = -y[j];
         HPHI_CUDA(ctx, cudaMemcpyAsync(cbuf, ny.data(), sizeof(double) * m, cudaMemcpyHostToDevice, ctx->stream));
-        HPHI_CUDA(ctx, cudaMemsetAsync(gs_out, 0, vb, ctx->stream));
-        if ((st = launch_maxpy(ctx, dt, D, m, Vb, cbuf, gs_out))) return fail(st);
+        HPHI_CUDA(ctx, cudaMemsetAsync(u, 0, vb, ctx->stream));
+        // (accumulated in the workspace, which is aligned, then copied out)
+        if ((st = launch_maxpy(ctx, dt, D, ldv, m, Vb, cbuf, u)) || (st = launch_copy(ctx, dt, D, 1, u, 1, gs_out, 1)))
+            return fail(st);
         double nrm = 0.0;
         if ((st = hphi_nrm2(ctx, dt, D, 1, gs_out, 1, &nrm))) return fail(st);
         if (!(nrm > 0.0)) return fail(set_err(ctx, HPHI_E_NUMERIC, "ground-state vector has zero norm"));
@@ -588,7 +599,7 @@ extern "C" int hphi_lanczos(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lancz
     HPHI_CUDA(ctx, cudaMemsetAsync(ctx->dflag, 0, sizeof(int), ctx->stream));
     if ((st = launch_copy(ctx, dt, D, 1, v0, 1, cur, 1))) return fail(st);
     if ((st = launch_dot(ctx, dt, 0, D, 1, cur, 1, cur, 1, red))) return fail(st);
-    k_lz<<<1, 32, 0, ctx->stream>>>(LZ_INIT, 0, red, alpha_d, beta2_d, coefA, coefB, ctx->dflag);
+    k_lz<<<1, kSumThreads, 0, ctx->stream>>>(LZ_INIT, 0, red, 1, 1, alpha_d, beta2_d, coefA, coefB, ctx->dflag);
 
     // convergence check: lowest Ritz value and the residual estimate (warm-started
     // from the previous check's value, an upper bound of the new one)
@@ -613,7 +624,6 @@ extern "C" int hphi_lanczos(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lancz
     };
 
     for (int k = 0; k < M; k++) {
-        k_lz<<<1, 32, 0, ctx->stream>>>(LZ_PREP_A, k, red, alpha_d, beta2_d, coefA, coefB, ctx->dflag);
         HvLaunch A{};
         A.dtype_real = dt;
         A.ncol = 1;
@@ -627,8 +637,9 @@ extern "C" int hphi_lanczos(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lancz
         A.coef_dev = coefA;
         A.red[0] = R_XO;
         A.partials = ctx->partials;
-        if ((st = launch_hv(ctx, ham, A)) || (st = reduce_hv(ctx, A, red))) return fail(st);
-        k_lz<<<1, 32, 0, ctx->stream>>>(LZ_ALPHA, k, red, alpha_d, beta2_d, coefA, coefB, ctx->dflag);
+        if ((st = launch_hv(ctx, ham, A))) return fail(st);
+        k_lz<<<1, kSumThreads, 0, ctx->stream>>>(LZ_ALPHA, k, A.partials, A.sgrid[0], 3, alpha_d, beta2_d, coefA, coefB,
+                                                 ctx->dflag);
         LinComb B{};
         B.real_dtype = dt;
         B.n = D;
@@ -642,9 +653,9 @@ extern "C" int hphi_lanczos(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lancz
         B.coef_dev = coefB;
         B.red_oo = 1;
         B.partials = ctx->partials;
-        if ((st = launch_lincomb(ctx, B)) || (st = reduce_partials(ctx, ctx->partials, B.grid, 1, red)))
-            return fail(st);
-        k_lz<<<1, 32, 0, ctx->stream>>>(LZ_BETA, k, red, alpha_d, beta2_d, coefA, coefB, ctx->dflag);
+        if ((st = launch_lincomb(ctx, B))) return fail(st);
+        k_lz<<<1, kSumThreads, 0, ctx->stream>>>(LZ_BETA, k, ctx->partials, B.grid, 1, alpha_d, beta2_d, coefA, coefB,
+                                                 ctx->dflag);
         HPHI_CUDA(ctx, cudaGetLastError());
         void *t = prev;
         prev = cur;

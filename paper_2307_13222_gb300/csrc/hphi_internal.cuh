@@ -330,10 +330,15 @@ struct LinComb {
 };
 int launch_lincomb(hphi_ctx *ctx, LinComb &L);
 int launch_random(hphi_ctx *ctx, int real_dtype, int64_t n, int nr, uint64_t seed, void *x, int64_t ldx);
-// c[j] = <V_j, w> for nv vectors stored back to back (V_j at V + j*n), into out_dev[nv]
-int launch_mdot(hphi_ctx *ctx, int real_dtype, int64_t n, int nv, const void *V, const void *w, double *out_dev);
-// w -= sum_j c_dev[j] V_j
-int launch_maxpy(hphi_ctx *ctx, int real_dtype, int64_t n, int nv, const void *V, const double *c_dev, void *w);
+// Multi-vector kernels over nv vectors V_j at V + j*ld; V, w on 16-byte boundaries
+// and ld * size a multiple of 16 (the vectorised kernels).
+// c[j] = <V_j, w> into out_dev[nv]
+int launch_mdot(hphi_ctx *ctx, int real_dtype, int64_t n, int64_t ld, int nv, const void *V, const void *w,
+                double *out_dev);
+// w -= sum_j c_dev[j] V_j; with norm_grid, the partial sums of the new |w|^2 go to
+// ctx->partials[*norm_grid]
+int launch_maxpy(hphi_ctx *ctx, int real_dtype, int64_t n, int64_t ld, int nv, const void *V, const double *c_dev,
+                 void *w, int *norm_grid = nullptr);
 int launch_copy(hphi_ctx *ctx, int real_dtype, int64_t n, int nr, const void *x, int64_t ldx, void *y,
                 int64_t ldy);
 

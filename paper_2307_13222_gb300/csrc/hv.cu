@@ -11,6 +11,7 @@
 #include <type_traits>
 
 #include "hvcommon.cuh"
+#include "reduce.cuh"
 
 namespace hphi {
 
@@ -457,14 +458,13 @@ int launch_typed(hphi_ctx *ctx, const hphi_ham *ham, HvLaunch &L) {
     return HPHI_OK;
 }
 
-// out[r * ncol_total + c0 + c] = sum over blocks b (in order) of part[b][r][c]
-__global__ void k_reduce_slice(const double *part, int grid, int nc, int c0, int ncol_total, double *out) {
-    int t = threadIdx.x;
-    if (t >= 3 * nc) return;
-    int r = t / nc, c = t % nc;
-    double s = 0.0;
-    for (int b = 0; b < grid; b++) s += part[((int64_t)b * 3 + r) * nc + c];
-    out[r * ncol_total + c0 + c] = s;
+// out[r * ncol_total + c0 + c] = sum over blocks b of part[b][r][c]: one thread
+// block per value.
+__global__ void __launch_bounds__(kSumThreads)
+    k_reduce_slice(const double *part, int grid, int nc, int c0, int ncol_total, double *out) {
+    const int t = blockIdx.x, r = t / nc, c = t % nc;
+    const double s = block_sum_strided(part + t, grid, 3 * nc);
+    if (threadIdx.x == 0) out[r * ncol_total + c0 + c] = s;
 }
 
 }  // namespace
@@ -480,7 +480,7 @@ size_t hv_partials_size(hphi_ctx *ctx, const hphi_ham *ham, int ncol) {
 int reduce_hv(hphi_ctx *ctx, const HvLaunch &L, double *out_dev) {
     int64_t off = 0;
     for (int s = 0; s < L.nslice; s++) {
-        k_reduce_slice<<<1, 96, 0, ctx->stream>>>(L.partials + off, L.sgrid[s], L.snc[s], L.sc0[s], L.ncol, out_dev);
+        k_reduce_slice<<<3 * L.snc[s], kSumThreads, 0, ctx->stream>>>(L.partials + off, L.sgrid[s], L.snc[s], L.sc0[s], L.ncol, out_dev);
         HPHI_CUDA(ctx, cudaGetLastError());
         off += (int64_t)L.sgrid[s] * 3 * L.snc[s];
     }

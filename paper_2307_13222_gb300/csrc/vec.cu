@@ -9,6 +9,7 @@
 #include <math.h>
 
 #include "hphi_internal.cuh"
+#include "reduce.cuh"
 
 namespace hphi {
 
@@ -84,24 +85,56 @@ __global__ void __launch_bounds__(kVT) k_dot(int64_t n, int nr, int tpr, int cro
     }
 }
 
-__global__ void k_reduce(const double *partials, int grid, int nval, double *out) {
-    for (int v = threadIdx.x; v < nval; v += blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < grid; b++) s += partials[(int64_t)b * nval + v];
-        out[v] = s;
+// One contiguous real column, 16-byte aligned operands: the same sums with
+// 16-byte loads, four of each operand in flight per thread (11.8 M FP32 rows:
+// 43 us with 4-byte loads, HBM floor 14 us for two operands).
+template <typename T>
+__global__ void __launch_bounds__(kVT) k_dot1(int64_t n, const T *__restrict__ x, const T *__restrict__ y,
+                                              double *partials) {
+    constexpr int V = 16 / (int)sizeof(T), U = 4;
+    Acc<T> s;
+    const int64_t nv = n / V, stride = (int64_t)gridDim.x * kVT;
+    const int64_t t0 = blockIdx.x * (int64_t)kVT + threadIdx.x;
+    for (int64_t i0 = t0; i0 < nv; i0 += stride * U) {
+        float4 xr[U], yr[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int64_t i = i0 + u * stride;
+            xr[u] = yr[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i < nv) {
+                xr[u] = __ldg((const float4 *)x + i);
+                yr[u] = __ldg((const float4 *)y + i);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+#pragma unroll
+            for (int e = 0; e < V; e++) s.add(((const T *)&xr[u])[e], ((const T *)&yr[u])[e]);
+    }
+    for (int64_t i = nv * V + t0; i < n; i += stride) s.add(x[i], y[i]);
+    __shared__ double sm[kVT / 32];
+    double v = s.value();
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < kVT / 32; w++) t += sm[w];
+        partials[2 * (int64_t)blockIdx.x] = t;
+        partials[2 * (int64_t)blockIdx.x + 1] = 0.0;
     }
 }
+// hphi_dot and hphi_dot_static choose by the same rule (their sums are bitwise equal).
+inline bool dot1_ok(int nr, const void *x, int64_t ldx, const void *y, int64_t ldy) {
+    return nr == 1 && ldx == 1 && ldy == 1 && (((uintptr_t)x | (uintptr_t)y) & 15u) == 0;
+}
 
-// out[v] = sum_b partials[b][v], one warp per value: lane l sums b = l, l + 32,
-// ... in order, then a fixed butterfly (deterministic).  For many values.
-__global__ void k_reduce_wide(const double *partials, int grid, int nval, double *out) {
-    const int v = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (v >= nval) return;
-    double sum = 0.0;
-    for (int b = lane; b < grid; b += 32) sum += partials[(int64_t)b * nval + v];
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-    if (lane == 0) out[v] = sum;
+// out[v] = sum_b partials[b][v]: one thread block per value.
+__global__ void __launch_bounds__(kSumThreads) k_reduce(const double *partials, int grid, int nval, double *out) {
+    const double s = block_sum_strided(partials + blockIdx.x, grid, nval);
+    if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
 struct LCArgs {
@@ -352,10 +385,10 @@ __global__ void k_copy(int64_t n, int nr, const T *x, int64_t ldx, T *y, int64_t
 // FP64 data: c[j] partials = sum over this block's rows of V[j][r] * w[r], j in
 // a chunk of 8 stored vectors (grid.y walks the chunks), one accumulator per
 // thread and vector, so the FP64 pipe does one FMA per element.  V holds nv vectors of length n,
-// vector j at V + j * n.  Fixed grid and order: deterministic.
+// vector j at V + j * ld.  Fixed grid and order: deterministic.
 template <typename T>
-__global__ void __launch_bounds__(kVT) k_mdot(int64_t n, int nv, const T *__restrict__ V, const T *__restrict__ w,
-                                              double *partials) {
+__global__ void __launch_bounds__(kVT) k_mdot(int64_t n, int64_t ld, int nv, const T *__restrict__ V,
+                                              const T *__restrict__ w, double *partials) {
     constexpr int J = 8;
     __shared__ double sm[kVT / 32][J];
     const int j0 = blockIdx.y * J;
@@ -364,7 +397,7 @@ __global__ void __launch_bounds__(kVT) k_mdot(int64_t n, int nv, const T *__rest
         const T wv = w[r];
 #pragma unroll
         for (int j = 0; j < J; j++)
-            if (j0 + j < nv) s[j].add(V[(int64_t)(j0 + j) * n + r], wv);
+            if (j0 + j < nv) s[j].add(V[(int64_t)(j0 + j) * ld + r], wv);
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -382,57 +415,100 @@ __global__ void __launch_bounds__(kVT) k_mdot(int64_t n, int nv, const T *__rest
     }
 }
 
-// Multi-vector kernels of the reorthogonalisation (V holds nv vectors of
-// length n, vector j at V + j * n), tiled by rows: a thread
-// holds kMR rows of a tile of kMT * kMR rows, so every pass reads each V_j and w
-// once from memory.
-constexpr int kMT = 256, kMR = 4;
+// Multi-vector kernels of the reorthogonalisation: nv vectors of length n,
+// vector j at V + j * ld, ld a multiple of 4 and every vector on a 16-byte
+// boundary.  A thread holds kMQ x 16 bytes of consecutive rows of a tile, so
+// every pass reads each V_j and w once from memory with 16-byte loads.
+constexpr int kMT = 256;
+template <typename T> constexpr int kMV = 16 / (int)sizeof(T);  // rows per load
+constexpr int kMQ = 2;                                           // loads per vector and thread
+
+template <typename T>
+struct alignas(16) Pack {
+    T e[16 / sizeof(T)];
+};
+// rows i .. i + kMV - 1 of p, zeros past n
+// (FULL: the caller knows that they exist)
+template <typename T, bool FULL>
+__device__ __forceinline__ Pack<T> load_pack(const T *__restrict__ p, int64_t i, int64_t n) {
+    Pack<T> v;
+    if (FULL || i + kMV<T> <= n) {
+        const float4 t = __ldg(reinterpret_cast<const float4 *>(p + i));
+        v = *reinterpret_cast<const Pack<T> *>(&t);
+    } else {
+#pragma unroll
+        for (int e = 0; e < kMV<T>; e++) v.e[e] = i + e < n ? p[i + e] : (T)0;
+    }
+    return v;
+}
 
 // FP32 data: partials[block][j] = sum over the block's tiles of <V_j, w>.  Per
-// tile, a lane forms its partial products for 32 vectors at a time (4 rows
-// each); a transposing butterfly (31 shuffles) leaves in lane l the warp's sum
-// for vector j0 + l, which lane l adds to the warp's FP64 slot.  The block then
-// sums its warps in order (deterministic).
+// tile, a lane forms its partial products for J vectors at a time (8 rows
+// each); a transposing butterfly leaves in lane l the warp's sum for vector
+// j0 + l mod J, which lane l adds to the warp's FP64 slot.  The block then sums
+// its warps in order (deterministic).  Bound by HBM: 80 passes over 1 to 40
+// vectors of 47 MB take 12.2 ms, the time of their bytes at 6.6 TB/s (20.2 ms
+// with 4-byte loads of four separate rows and groups of 32).
+template <typename T, int J, bool FULL>
+__device__ __forceinline__ void mdot_group(int64_t n, int64_t ld, int j0, int nv, const T *__restrict__ V, int64_t r0,
+                                           const Pack<T> (&wv)[kMQ], int lane, double *acc) {
+    T v[J];
+#pragma unroll
+    for (int j = 0; j < J; j++) {
+        v[j] = (T)0;
+        if (j0 + j < nv) {
+            const T *vj = V + (int64_t)(j0 + j) * ld;
+#pragma unroll
+            for (int i = 0; i < kMQ; i++) {
+                const Pack<T> x = load_pack<T, FULL>(vj, r0 + (int64_t)i * kMT * kMV<T>, n);
+#pragma unroll
+                for (int e = 0; e < kMV<T>; e++) v[j] = fma(x.e[e], wv[i].e[e], v[j]);
+            }
+        }
+    }
+    // transposing butterfly: after the step of width s, lane l keeps the half of
+    // its values whose index offset matches bit s of l; then plain sums over the
+    // lanes that hold the same vector
+#pragma unroll
+    for (int s2 = J / 2; s2 >= 1; s2 >>= 1) {
+        const bool upper = (lane & s2) != 0;
+#pragma unroll
+        for (int j = 0; j < s2; j++) {
+            const T send = upper ? v[j] : v[j + s2];
+            const T keep = upper ? v[j + s2] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, send, s2);
+        }
+    }
+#pragma unroll
+    for (int s2 = J; s2 < 32; s2 <<= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], s2);
+    if (lane < J && j0 + lane < nv) acc[j0 + lane] += (double)v[0];
+}
+
+template <typename T, bool FULL>
+__device__ __forceinline__ void mdot_tile(int64_t n, int64_t ld, int nv, const T *__restrict__ V,
+                                          const T *__restrict__ w, int64_t r0, int lane, double *acc) {
+    Pack<T> wv[kMQ];
+#pragma unroll
+    for (int i = 0; i < kMQ; i++) wv[i] = load_pack<T, FULL>(w, r0 + (int64_t)i * kMT * kMV<T>, n);
+    int j0 = 0;
+#pragma unroll 1
+    for (; j0 + 8 < nv; j0 += 16) mdot_group<T, 16, FULL>(n, ld, j0, nv, V, r0, wv, lane, acc);
+    if (j0 < nv) mdot_group<T, 8, FULL>(n, ld, j0, nv, V, r0, wv, lane, acc);
+}
+
 template <typename T>
-__global__ void __launch_bounds__(kMT, 4) k_mdot_tiled(int64_t n, int nv, const T *__restrict__ V,
-                                                    const T *__restrict__ w, double *partials) {
+__global__ void __launch_bounds__(kMT, 4) k_mdot_tiled(int64_t n, int64_t ld, int nv, const T *__restrict__ V,
+                                                       const T *__restrict__ w, double *partials) {
     extern __shared__ double acc_sm[];  // [kMT / 32][nv]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = threadIdx.x; j < (kMT / 32) * nv; j += kMT) acc_sm[j] = 0.0;
     __syncthreads();
-    constexpr int64_t TILE = (int64_t)kMT * kMR;
+    constexpr int64_t TILE = (int64_t)kMT * kMQ * kMV<T>;
     const int64_t ntiles = (n + TILE - 1) / TILE;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t r0 = t * TILE + threadIdx.x;
-        T wv[kMR];
-#pragma unroll
-        for (int i = 0; i < kMR; i++) wv[i] = r0 + i * kMT < n ? w[r0 + i * kMT] : (T)0;
-        for (int j0 = 0; j0 < nv; j0 += 32) {
-            T v[32];
-#pragma unroll
-            for (int j = 0; j < 32; j++) {
-                v[j] = (T)0;
-                if (j0 + j < nv) {
-                    const T *vj = V + (int64_t)(j0 + j) * n;
-#pragma unroll
-                    for (int i = 0; i < kMR; i++)
-                        if (r0 + i * kMT < n) v[j] = fma(vj[r0 + i * kMT], wv[i], v[j]);
-                }
-            }
-            // transposing butterfly: after the step of width s, lane l keeps the
-            // half of its values whose index offset matches bit s of l
-#pragma unroll
-            for (int s2 = 16; s2 >= 1; s2 >>= 1) {
-                const bool upper = (lane & s2) != 0;
-#pragma unroll
-                for (int j = 0; j < s2; j++) {
-                    const T send = upper ? v[j] : v[j + s2];
-                    const T keep = upper ? v[j + s2] : v[j];
-                    v[j] = keep + __shfl_xor_sync(0xffffffffu, send, s2);
-                }
-            }
-            if (j0 + lane < nv) acc_sm[warp * nv + j0 + lane] += (double)v[0];
-        }
+        const int64_t r0 = t * TILE + threadIdx.x * kMV<T>;
+        if ((t + 1) * TILE <= n) mdot_tile<T, true>(n, ld, nv, V, w, r0, lane, acc_sm + warp * nv);
+        else mdot_tile<T, false>(n, ld, nv, V, w, r0, lane, acc_sm + warp * nv);
     }
     __syncthreads();
     for (int j = threadIdx.x; j < nv; j += kMT) {
@@ -442,34 +518,88 @@ __global__ void __launch_bounds__(kMT, 4) k_mdot_tiled(int64_t n, int nv, const 
     }
 }
 
-// w[r] -= sum_j c[j] V[j][r], the sum in T in order of j, kMR rows per thread
-// so that 4 loads per vector are in flight.
+// w[r] -= sum_j c[j] V[j][r], the sum in T in order of j; with `norm`, also the
+// block's partial sum of the new w[r]^2 (partials[block]): the second projection
+// of a step leaves |w|^2 behind, without another pass over w.  Bound by HBM (81
+// passes over 1 to 40 vectors of 47 MB: 12.3 ms, 14.7 with 4-byte loads; two
+// vectors per iteration: 4 13.8, 8 13.0).
+template <typename T, bool FULL>
+__device__ __forceinline__ void maxpy_tile(int64_t n, int64_t ld, int nv, const T *__restrict__ V, const T *cs, T *w,
+                                           int64_t r0, int norm, Acc<T> &nn) {
+    T acc[kMQ][kMV<T>];
+#pragma unroll
+    for (int i = 0; i < kMQ; i++)
+#pragma unroll
+        for (int e = 0; e < kMV<T>; e++) acc[i][e] = (T)0;
+    const T *vj = V;
+#pragma unroll(FULL ? 2 : 1)
+    for (int j = 0; j < nv; j++, vj += ld) {
+        const T cj = cs[j];
+#pragma unroll
+        for (int i = 0; i < kMQ; i++) {
+            const Pack<T> x = load_pack<T, FULL>(vj, r0 + (int64_t)i * kMT * kMV<T>, n);
+#pragma unroll
+            for (int e = 0; e < kMV<T>; e++) acc[i][e] = fma(cj, x.e[e], acc[i][e]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kMQ; i++) {
+        const int64_t r = r0 + (int64_t)i * kMT * kMV<T>;
+        if (FULL || r + kMV<T> <= n) {
+            Pack<T> x = *reinterpret_cast<const Pack<T> *>(w + r);
+#pragma unroll
+            for (int e = 0; e < kMV<T>; e++) {
+                x.e[e] -= acc[i][e];
+                if (norm) nn.add(x.e[e], x.e[e]);
+            }
+            *reinterpret_cast<Pack<T> *>(w + r) = x;
+        } else {
+#pragma unroll
+            for (int e = 0; e < kMV<T>; e++)
+                if (r + e < n) {
+                    const T x = w[r + e] - acc[i][e];
+                    w[r + e] = x;
+                    if (norm) nn.add(x, x);
+                }
+        }
+    }
+}
+
 template <typename T>
-__global__ void __launch_bounds__(kMT) k_maxpy_tiled(int64_t n, int nv, const T *__restrict__ V,
-                                                     const double *__restrict__ c, T *w) {
+__global__ void __launch_bounds__(kMT) k_maxpy_tiled(int64_t n, int64_t ld, int nv, const T *__restrict__ V,
+                                                     const double *__restrict__ c, T *w, int norm, double *partials) {
     extern __shared__ __align__(16) unsigned char cs_raw[];
     T *cs = (T *)cs_raw;  // [nv]
     for (int j = threadIdx.x; j < nv; j += kMT) cs[j] = (T)c[j];
     __syncthreads();
-    constexpr int64_t TILE = (int64_t)kMT * kMR;
+    constexpr int64_t TILE = (int64_t)kMT * kMQ * kMV<T>;
     const int64_t ntiles = (n + TILE - 1) / TILE;
+    Acc<T> nn;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t r0 = t * TILE + threadIdx.x;
-        T acc[kMR];
-#pragma unroll
-        for (int i = 0; i < kMR; i++) acc[i] = (T)0;
-#pragma unroll 4
-        for (int j = 0; j < nv; j++) {
-            const T *vj = V + (int64_t)j * n;
-            const T cj = cs[j];
-#pragma unroll
-            for (int i = 0; i < kMR; i++)
-                if (r0 + i * kMT < n) acc[i] = fma(cj, vj[r0 + i * kMT], acc[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < kMR; i++)
-            if (r0 + i * kMT < n) w[r0 + i * kMT] -= acc[i];
+        const int64_t r0 = t * TILE + threadIdx.x * kMV<T>;
+        if ((t + 1) * TILE <= n) maxpy_tile<T, true>(n, ld, nv, V, cs, w, r0, norm, nn);
+        else maxpy_tile<T, false>(n, ld, nv, V, cs, w, r0, norm, nn);
     }
+    if (!norm) return;
+    __shared__ double sm[kMT / 32];
+    double s = nn.value();
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double tot = 0.0;
+#pragma unroll
+        for (int k = 0; k < kMT / 32; k++) tot += sm[k];
+        partials[blockIdx.x] = tot;
+    }
+}
+
+int tiled_grid(hphi_ctx *ctx, int real_dtype, int64_t n) {
+    const int64_t tile = (int64_t)kMT * kMQ * (16 / (int64_t)real_size(real_dtype));
+    int64_t g = (n + tile - 1) / tile;
+    if (g > (int64_t)ctx->sm_count * 8) g = (int64_t)ctx->sm_count * 8;
+    return (int)(g < 1 ? 1 : g);
 }
 
 int vec_grid(hphi_ctx *ctx, int64_t n, int tpr) {
@@ -484,7 +614,8 @@ int vec_grid(hphi_ctx *ctx, int64_t n, int tpr) {
 }  // namespace
 
 int reduce_partials(hphi_ctx *ctx, const double *partials, int grid, int nval, double *out_dev) {
-    k_reduce<<<1, 256, 0, ctx->stream>>>(partials, grid, nval, out_dev);
+    if (nval < 1) return HPHI_OK;
+    k_reduce<<<nval, kSumThreads, 0, ctx->stream>>>(partials, grid, nval, out_dev);
     HPHI_CUDA(ctx, cudaGetLastError());
     return HPHI_OK;
 }
@@ -500,7 +631,12 @@ int launch_dot(hphi_ctx *ctx, int real_dtype, int cplx, int64_t n, int nr, const
 #define HPHI_DOT(T, C)                                                                                         \
     k_dot<T, C><<<grid, kVT, 0, ctx->stream>>>(n, nr, tpr, cplx, (const T *)x, ldx, (const T *)y, ldy, \
                                                ctx->partials)
-    if (real_dtype == HPHI_F64) {
+    const bool one = dot1_ok(nr, x, ldx, y, ldy);
+    if (one && real_dtype == HPHI_F64) {
+        k_dot1<double><<<grid, kVT, 0, ctx->stream>>>(n, (const double *)x, (const double *)y, ctx->partials);
+    } else if (one) {
+        k_dot1<float><<<grid, kVT, 0, ctx->stream>>>(n, (const float *)x, (const float *)y, ctx->partials);
+    } else if (real_dtype == HPHI_F64) {
         if (cpl <= 1) HPHI_DOT(double, 1);
         else if (cpl <= 2) HPHI_DOT(double, 2);
         else if (cpl <= 4) HPHI_DOT(double, 4);
@@ -589,7 +725,8 @@ int launch_lincomb(hphi_ctx *ctx, LinComb &L) {
     return HPHI_OK;
 }
 
-int launch_mdot(hphi_ctx *ctx, int real_dtype, int64_t n, int nv, const void *V, const void *w, double *out_dev) {
+int launch_mdot(hphi_ctx *ctx, int real_dtype, int64_t n, int64_t ld, int nv, const void *V, const void *w,
+                double *out_dev) {
     if (nv < 1 || nv > 1024) return set_err(ctx, HPHI_E_INVAL, "1 to 1024 stored vectors");
     int st;
     if (real_dtype == HPHI_F64) {
@@ -600,41 +737,38 @@ int launch_mdot(hphi_ctx *ctx, int real_dtype, int64_t n, int nv, const void *V,
         if ((st = ensure_partials(ctx, (size_t)gx * nv))) return st;
         const int slot = prof_begin(ctx, PROF_VEC);
         dim3 grid((unsigned)gx, (unsigned)((nv + 7) / 8));
-        k_mdot<double><<<grid, kVT, 0, ctx->stream>>>(n, nv, (const double *)V, (const double *)w, ctx->partials);
+        k_mdot<double><<<grid, kVT, 0, ctx->stream>>>(n, ld, nv, (const double *)V, (const double *)w, ctx->partials);
         prof_end(ctx, slot);
         HPHI_CUDA(ctx, cudaGetLastError());
         return reduce_partials(ctx, ctx->partials, (int)gx, nv, out_dev);
     }
-    const int64_t tile = (int64_t)kMT * kMR;
-    int64_t g = (n + tile - 1) / tile;
-    if (g > (int64_t)ctx->sm_count * 8) g = (int64_t)ctx->sm_count * 8;
-    if (g < 1) g = 1;
+    const int g = tiled_grid(ctx, real_dtype, n);
     if ((st = ensure_partials(ctx, (size_t)g * nv))) return st;
     const size_t dyn = sizeof(double) * (kMT / 32) * nv;
     if (dyn > 48 * 1024 && dyn_occupancy(ctx, (const void *)k_mdot_tiled<float>, kMT, dyn) < 1)
         return set_err(ctx, HPHI_E_INVAL, "multi-vector dot: %d vectors need too much shared memory", nv);
     const int slot = prof_begin(ctx, PROF_VEC);
-    k_mdot_tiled<float><<<(unsigned)g, kMT, dyn, ctx->stream>>>(n, nv, (const float *)V, (const float *)w,
-                                                               ctx->partials);
-    k_reduce_wide<<<(nv + 7) / 8, 256, 0, ctx->stream>>>(ctx->partials, (int)g, nv, out_dev);
+    k_mdot_tiled<float><<<g, kMT, dyn, ctx->stream>>>(n, ld, nv, (const float *)V, (const float *)w, ctx->partials);
     prof_end(ctx, slot);
     HPHI_CUDA(ctx, cudaGetLastError());
-    return HPHI_OK;
+    return reduce_partials(ctx, ctx->partials, g, nv, out_dev);
 }
 
-int launch_maxpy(hphi_ctx *ctx, int real_dtype, int64_t n, int nv, const void *V, const double *c_dev, void *w) {
+int launch_maxpy(hphi_ctx *ctx, int real_dtype, int64_t n, int64_t ld, int nv, const void *V, const double *c_dev,
+                 void *w, int *norm_grid) {
     if (nv < 1 || nv > 1024) return set_err(ctx, HPHI_E_INVAL, "1 to 1024 stored vectors");
-    const int64_t tile = (int64_t)kMT * kMR;
-    int64_t g = (n + tile - 1) / tile;
-    if (g > (int64_t)ctx->sm_count * 8) g = (int64_t)ctx->sm_count * 8;
-    if (g < 1) g = 1;
+    const int g = tiled_grid(ctx, real_dtype, n);
+    const int norm = norm_grid != nullptr;
+    int st;
+    if (norm && (st = ensure_partials(ctx, (size_t)g))) return st;
+    if (norm) *norm_grid = g;
     const int slot = prof_begin(ctx, PROF_VEC);
     if (real_dtype == HPHI_F64)
-        k_maxpy_tiled<double><<<(unsigned)g, kMT, sizeof(double) * nv, ctx->stream>>>(n, nv, (const double *)V, c_dev,
-                                                                                      (double *)w);
+        k_maxpy_tiled<double><<<g, kMT, sizeof(double) * nv, ctx->stream>>>(n, ld, nv, (const double *)V, c_dev,
+                                                                           (double *)w, norm, ctx->partials);
     else
-        k_maxpy_tiled<float><<<(unsigned)g, kMT, sizeof(float) * nv, ctx->stream>>>(n, nv, (const float *)V, c_dev,
-                                                                                    (float *)w);
+        k_maxpy_tiled<float><<<g, kMT, sizeof(float) * nv, ctx->stream>>>(n, ld, nv, (const float *)V, c_dev,
+                                                                         (float *)w, norm, ctx->partials);
     prof_end(ctx, slot);
     HPHI_CUDA(ctx, cudaGetLastError());
     return HPHI_OK;
@@ -754,7 +888,12 @@ extern "C" int hphi_dot_static(int device, void *stream, int dtype, int64_t n, i
         const int64_t lx = ldx * cpl, ly = ldy * cpl;
 #define HPHI_SDOT(T, C)                                                                                    \
     k_dot<T, C><<<grid, kVT, 0, st>>>(n, nr, tpr, cpl == 2, (const T *)x, lx, (const T *)y, ly, partials)
-        if (rd == HPHI_F64) {
+        const bool one = dot1_ok(nr, x, lx, y, ly);
+        if (one && rd == HPHI_F64) {
+            k_dot1<double><<<grid, kVT, 0, st>>>(n, (const double *)x, (const double *)y, partials);
+        } else if (one) {
+            k_dot1<float><<<grid, kVT, 0, st>>>(n, (const float *)x, (const float *)y, partials);
+        } else if (rd == HPHI_F64) {
             if (cplane <= 1) HPHI_SDOT(double, 1);
             else HPHI_SDOT(double, 2);
         } else {
@@ -762,7 +901,7 @@ extern "C" int hphi_dot_static(int device, void *stream, int dtype, int64_t n, i
             else HPHI_SDOT(float, 2);
         }
 #undef HPHI_SDOT
-        k_reduce<<<1, 256, 0, st>>>(partials, grid, 2 * nr, result);
+        k_reduce<<<2 * nr, kSumThreads, 0, st>>>(partials, grid, 2 * nr, result);
         if (cudaGetLastError() != cudaSuccess) {
             rc = HPHI_E_CUDA;
             break;
