@@ -63,7 +63,7 @@ int ensure_dscal(hphi_ctx *ctx, size_t n) {
 int dyn_occupancy(hphi_ctx *ctx, const void *fn, int threads, size_t dyn) {
     static std::mutex mu;
     static std::map<std::pair<const void *, int>, size_t> limit;              // raised limit per (kernel, device)
-    static std::map<std::tuple<const void *, int, size_t>, int> occupancy;  // per (kernel, device, size)
+    static std::map<std::tuple<const void *, int, int, size_t>, int> occupancy;  // per (kernel, device, threads, size)
     std::lock_guard<std::mutex> lk(mu);
     const int dev = ctx->device;
     auto key = std::make_pair(fn, dev);
@@ -84,7 +84,7 @@ int dyn_occupancy(hphi_ctx *ctx, const void *fn, int threads, size_t dyn) {
         it = limit.emplace(key, mx).first;
     }
     if (dyn > it->second) return 0;
-    auto ok = std::make_tuple(fn, dev, dyn);
+    auto ok = std::make_tuple(fn, dev, threads, dyn);
     auto jt = occupancy.find(ok);
     if (jt != occupancy.end()) return jt->second;
     int n = 0;

@@ -145,7 +145,9 @@ void free_ham(hphi_ham *h) {
     cudaFree(h->rowstate);
     cudaFree(h->seg_so);
     cudaFree(h->warp_tab);
+    cudaFree(h->hub_tab);
     delete h->warp;
+    delete h->hub;
     for (int p = 0; p < 2; p++) {
         cudaFree(h->tile_tab[p]);
         cudaFree(h->tile_diag[p]);
@@ -517,6 +519,7 @@ extern "C" int hphi_build_hamiltonian(hphi_ctx *ctx, const hphi_basis *basis, co
             if (e != cudaSuccess) st = cuda_err(ctx, e, "k_pack_ll");
         }
     }
+    if (!st) st = build_hub_tables(ctx, H);
     if (st) {
         free_ham(H);
         return st;

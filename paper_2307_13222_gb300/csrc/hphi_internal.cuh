@@ -127,6 +127,20 @@ struct WarpArgs {
     const unsigned char *img32, *img64;  // device: the tables' images (hv_warp.cu, WarpLayout)
 };
 
+// Hubbard kernel (hv_hub.cu): sizes and the fixed-point diagonal.
+struct HubV {        // V n_i n_j
+    int i, j;
+    long long v;
+};
+struct HubArgs {
+    int N, up_pad, ngrp, nv;      // up_pad: most up hops of a string, padded to 8
+    uint32_t nh, ddn;             // up and down strings
+    double scale64, scale32;      // fixed point to value
+    const long long *ufix;        // device [32]: U per site
+    const HubV *vfix;             // device [nv]
+    const long long *dup, *ddnf;  // device: V terms of one species alone, per up / down string (null: none)
+};
+
 // Lin tables of one species (spin string, or up / down fermion string).
 struct Species {
     int N = 0, n = 0, nlo = 0, nhi = 0;
@@ -222,6 +236,9 @@ struct hphi_ham {
     // available) and its device tables
     hphi::WarpArgs *warp = nullptr;
     unsigned char *warp_tab = nullptr;
+    // Hubbard kernel: its arguments (null when not available) and device tables
+    hphi::HubArgs *hub = nullptr;
+    long long *hub_tab = nullptr;
     // tiled block kernel (full space, 32 columns), per precision [0: FP32, 1: FP64]
     // (the tiles follow the row size): built on first use
     hphi::TileArgs *tile[2] = {nullptr, nullptr};
@@ -354,6 +371,8 @@ int lowest_ritz_warm(int m, const double *alpha, const double *beta2, double *wa
 int build_seg_tables(hphi_ctx *ctx, hphi_ham *H);
 // ---- segment kernel tables (hv_warp.cu) ----------------------------------------------
 int build_warp_tables(hphi_ctx *ctx, hphi_ham *H);
+// ---- Hubbard kernel tables (hv_hub.cu) -------------------------------------------------
+int build_hub_tables(hphi_ctx *ctx, hphi_ham *H);
 // ---- tiled block kernel tables (hv_tile.cu) ------------------------------------------
 int build_tile_tables(hphi_ctx *ctx, hphi_ham *H, int prec);
 

@@ -42,6 +42,7 @@
 // segment bits 6x5 3.66, 8 bits 5.68 (lanes idle in short segments); 8 uniform
 // loads in flight per lane 3.27, 16: 2.87, 24: 2.79; 16 mixed loads 3.32; two
 // batches in flight at a time 5.9 (spills at 64 registers); 16 warps per SM 3.4.
+#include "fixed.cuh"
 #include "hvcommon.cuh"
 
 #include <math.h>
@@ -58,21 +59,8 @@ namespace {
 constexpr int kLoadsU = 24, kLoadsM = 8;  // loads per lane in flight: uniform bonds, mixed bonds
 // threads per block: one block per SM, registers for 32 (FP64: 16) warps
 template <typename T> constexpr int kSegThreads = sizeof(T) == 4 ? 1024 : 512;
-constexpr int kFixShift = 29;  // 64-bit to 32-bit fixed point (the diagonal is below 2^59 in 64 bits)
 constexpr int kSegStage = 256;  // staged values per warp (a slot behind every segment stays 0)
 constexpr int kSegRows = 8;   // rows of a lane held in registers (C(10, 5) = 252 rows per segment)
-
-template <typename T>
-struct FixInt { using type = int; };
-template <>
-struct FixInt<double> { using type = long long; };
-
-// A 64-bit fixed-point value in T's fixed point (FP32: its upper 32 bits, rounded).
-template <typename T>
-inline typename FixInt<T>::type to_fix(long long v) {
-    if constexpr (sizeof(T) == 4) return (int)((v + (1ll << (kFixShift - 1))) >> kFixShift);
-    else return v;
-}
 
 // A bond of the image, in T's precision.
 struct WarpBond {     // a bond as the builder collects it
@@ -141,10 +129,7 @@ template <int NC>
 __device__ __forceinline__ void fma_rows(float c, const float (&v)[NC], float (&acc)[NC]) {
 #pragma unroll
     for (int i = 0; i + 1 < NC; i += 2)
-        asm("{.reg .b64 a, b, d; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %4}; mov.b64 d, {%0, %1};\n\t"
-            "fma.rn.f32x2 d, a, b, d; mov.b64 {%0, %1}, d;}"
-            : "+f"(acc[i]), "+f"(acc[i + 1])
-            : "f"(v[i]), "f"(v[i + 1]), "f"(c));
+        fma2(acc[i], acc[i + 1], c, v[i], v[i + 1]);
     if constexpr (NC % 2) acc[NC - 1] = fma(c, v[NC - 1], acc[NC - 1]);
 }
 template <int NC>

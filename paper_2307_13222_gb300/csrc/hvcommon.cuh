@@ -225,6 +225,9 @@ uint32_t staged_block_len(const hphi_ham *ham);
 // tiled two-pass block kernel (hv_tile.cu): full space, 32 columns (FP32 or FP64)
 template <typename T>
 int launch_tile(hphi_ctx *ctx, const hphi_ham *ham, HvArgs<T> &a, int red_mode, int *grid);
+// Hubbard kernel (hv_hub.cu): one column or one pair of columns
+template <typename T>
+int launch_hub(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int red_mode, int *grid);
 // segment kernel (hv_warp.cu): spin sector, one column
 template <typename T>
 int launch_warp(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int red_mode, int *grid);

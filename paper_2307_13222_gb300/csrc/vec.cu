@@ -461,8 +461,10 @@ __device__ __forceinline__ void mdot_group(int64_t n, int64_t ld, int j0, int nv
 #pragma unroll
             for (int i = 0; i < kMQ; i++) {
                 const Pack<T> x = load_pack<T, FULL>(vj, r0 + (int64_t)i * kMT * kMV<T>, n);
+                T p = x.e[0] * wv[i].e[0];
 #pragma unroll
-                for (int e = 0; e < kMV<T>; e++) v[j] = fma(x.e[e], wv[i].e[e], v[j]);
+                for (int e = 1; e < kMV<T>; e++) p = fma(x.e[e], wv[i].e[e], p);
+                v[j] += p;
             }
         }
     }

@@ -1,0 +1,94 @@
+"""Hubbard H*x kernel (one column, or one pair of columns; the automatic choice
+there) against the oracle and the generic kernel: numbers of up strings that
+are no multiple of the strings per thread block, one down string, thread-block
+sizes on both sides of their limits, V terms, hops of one species, the pair
+swap and the reductions.  FP64 1e-13, FP32 2e-6 of max|y|, as the other kernels."""
+import random
+
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import pair, rel_err
+from paper_2307_13222_gb300 import hphi
+from workloads import chain, hubbard_terms, random_vectors, square
+
+pytestmark = pytest.mark.gpu
+
+TOL = {torch.float64: 1e-13, torch.float32: 2e-6, torch.complex128: 1e-13, torch.complex64: 2e-6}
+
+
+def _terms(N, bonds, seed):
+    rng = random.Random(seed)
+    t = [("HOP", i, j, rng.choice([-1, -1, 0, 1]), rng.uniform(0.5, 1.5), 0.0) for i, j in bonds]
+    t += [("HUBBARD_U", i, i, 0, rng.uniform(-2, 8), 0.0) for i in range(N)]
+    return t + [("DENS_DENS", i, j, 0, rng.uniform(-1, 1), 0.0) for i, j in bonds[::2]]
+
+
+# (sites, up, down): 1 up or down string; 5, 6, 9 up strings; D_dn = 495 .. 792 (64 and 256
+# threads), 6435 (1024)
+@pytest.mark.parametrize("lx,ly,nu,nd", [(5, 1, 1, 0), (5, 1, 0, 2), (4, 1, 2, 2), (9, 1, 8, 4), (6, 2, 1, 4),
+                                         (6, 2, 11, 5), (5, 3, 1, 7), (7, 1, 3, 4)])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32, torch.complex128, torch.complex64])
+def test_hubbard_kernel(lx, ly, nu, nd, dtype):
+    N = lx * ly
+    m, b, h = pair("HUBBARD", N, nu, nd, _terms(N, square(lx, ly) if ly > 1 else chain(lx), N * 7 + nu))
+    cplx = dtype.is_complex
+    x = torch.from_numpy(random_vectors(m.dim, 1, N, complex_=cplx, normalize=False)[:, 0].copy()).to(dtype)
+    y = torch.from_numpy(random_vectors(m.dim, 1, N + 1, complex_=cplx, normalize=False)[:, 0].copy()).to(dtype)
+    for alpha, beta in ((0.8, 0.0), (-1.1, 0.35)):
+        pad = torch.full((m.dim + 2,), float("nan"), dtype=dtype, device="cuda")
+        xd = pad.clone()[1:1 + m.dim].copy_(x)
+        yd = pad[1:1 + m.dim].copy_(y)
+        hphi.hphi_apply_H(h, xd, yd, alpha, beta)
+        assert h.ctx.last_kernel().startswith("k_hub<")
+        f = torch.float64
+        if cplx:
+            xr, yr = torch.view_as_real(x).to(f).numpy(), torch.view_as_real(y).to(f).numpy()
+            want = sum(u * m.apply(np.ascontiguousarray(xr[:, k]), alpha, beta, np.ascontiguousarray(yr[:, k]))
+                       for k, u in ((0, 1.0), (1, 1j)))
+        else:
+            want = m.apply(x.to(f).numpy(), alpha, beta, y.to(f).numpy().copy())
+        assert rel_err(yd.cpu().numpy(), want) < TOL[dtype]
+        assert pad[:1].isnan().all() and pad[1 + m.dim:].isnan().all()
+        h.set_tuning(variant=0)
+        y0 = y.cuda()
+        hphi.hphi_apply_H(h, xd, y0, alpha, beta)
+        assert rel_err(yd.cpu().numpy(), y0.cpu().numpy()) < TOL[dtype]
+        h.set_tuning(variant=-1)
+
+
+def _h(m, x):
+    return m.apply(np.ascontiguousarray(x.real)) + 1j * m.apply(np.ascontiguousarray(x.imag))
+
+
+@pytest.mark.parametrize("dtype", [torch.complex128, torch.complex64])
+def test_hubbard_kernel_pair_swap_and_reductions(dtype):
+    """Real-time and cTPQ steps of one complex column (pair swap, fused
+    reductions), and Lanczos scalars of one real column."""
+    m, b, h = pair("HUBBARD", 8, 4, 3, hubbard_terms(8, chain(8), t=1.0, U=4.0, V=0.3))
+    tol = 1e-12 if dtype == torch.complex128 else 2e-5
+    V0 = random_vectors(m.dim, 1, 5, complex_=True)
+    Vg = torch.from_numpy(V0[:, 0].copy()).to(dtype).cuda()
+    Vo = V0.copy()
+    for _ in range(4):
+        n2, e, h2, n2n = hphi.hphi_time_step(h, Vg, 0.02, 6)
+        no, eo, noo = m.time_step(Vo, 0.02, 6)
+    assert h.ctx.last_kernel().startswith("k_hub<")
+    assert rel_err(Vg.cpu().numpy(), Vo[:, 0]) < tol
+    assert np.allclose(n2, no, rtol=tol) and np.allclose(e, eo, rtol=10 * tol) and np.allclose(n2n, noo, rtol=tol)
+    assert abs(h2[0] - np.linalg.norm(_h(m, Vo[:, 0])) ** 2) < 1e-3 * h2[0]  # conserved to the step's order
+    norm2 = np.zeros(1)
+    Wg = torch.from_numpy(V0[:, 0].copy()).to(dtype).cuda()
+    Wo = V0.copy()
+    for _ in range(3):
+        e, h2, logd = hphi.hphi_tpq_step(h, Wg, 0.05, 4, norm2)
+        eo, h2o, do = m.tpq_step(Wo, 0.05, 4)
+        assert np.allclose(e, eo, rtol=10 * tol) and np.allclose(h2, h2o, rtol=10 * tol)
+        assert np.allclose(logd, np.log(do), atol=10 * tol)
+    rd = torch.float64 if dtype == torch.complex128 else torch.float32
+    v0 = np.ascontiguousarray(V0[:, 0].real)
+    got = hphi.hphi_lanczos(h, torch.from_numpy(v0).to(rd).cuda(), 10, 0.0, 10)
+    want = m.lanczos(v0, 10, 0.0)
+    assert np.allclose(got["alpha"], want["alpha"], atol=10 * tol) and np.allclose(got["beta"], want["beta"][1:],
+                                                                                   atol=10 * tol)
