@@ -72,14 +72,23 @@ struct DTerm {
 };
 
 // Tiled two-pass block H*V (hv_tile.cu): per pass the bit set of the tile's
-// rows (nin bits varied inside a tile, nout bits fixed per tile), its bonds
-// (masks and Jxy/2), and the bit-deposit tables of both index parts.
+// rows (nin bits varied inside a tile, nout bits fixed per tile), the bonds as
+// entries over items, the item bits (as row offsets), and the bit-deposit tables
+// of both index parts.
 constexpr int kTileMaxBonds = 64;
+struct TileEnt {
+    uint32_t mo;     // the bond's sites outside the item
+    int32_t d0, d1;  // target row - (row ^ mo): first site of mo up / otherwise
+    uint32_t mask;   // rows and lane groups it applies to: mo up | otherwise << 8
+    double c;        // Jxy/2
+};
 struct TileArgs {
     const uint32_t *tab;  // [2 passes][inner, outer][4 bytes][256]
-    int nin[2], nout[2], nb[2];
-    uint32_t m[2][kTileMaxBonds];
-    double c[2][kTileMaxBonds];
+    const TileEnt *ent[2];
+    int nin[2], nout[2];
+    int ne[2], nfull[2];  // entries; those without a site in the item come first
+    int site[2][4];       // 2^site of the item bits: lane groups, then register rows
+    unsigned *ticket[2];  // next pair of items of a pass (null: fixed stride)
 };
 
 // Per-Hamiltonian descriptor (device copy read by every block at set-up).
@@ -171,6 +180,7 @@ struct hphi_ctx {
     // driver vectors (Lanczos / TPQ), grown on demand
     void *vec[4] = {nullptr, nullptr, nullptr, nullptr};
     size_t vec_bytes = 0;
+    unsigned *ticket = nullptr;  // item counters of the tiled kernel's passes
     int *dflag = nullptr;        // device status word of consistency checks
     // high-high pass: its partial products when y cannot hold them
     void *seg_tmp = nullptr;
