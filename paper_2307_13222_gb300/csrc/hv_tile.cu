@@ -29,15 +29,15 @@
 // v != y), else in a context buffer.
 //
 // Inside a pass, a warp owns an item: the rows that share all bits but the
-// lowest item bits of S_k (16 rows in FP32, 8 in FP64; 16 bytes of a row per
-// lane, 4 rows per lane).  What a bond does to an item is decided once, one bond
+// first item bits of S_k (16 rows in FP32, 4 per lane, 16 bytes of a row per lane;
+// 8 in FP64, all in every lane, one column per lane).  What a bond does to an item is decided once, one bond
 // per lane: with both sites outside the item it applies to all its rows or to
 // none; with one site inside, to the rows whose bit is the opposite of the other
 // site's; with both inside, to the rows where the two differ, in two parts.  In
 // every case the target rows lie at one fixed row offset, so an applicable bond
 // is an entry (first target row, coefficient, masks of the rows and lane groups
-// it touches) of the warp's list, and costs one address, 4 16-byte loads and
-// their FMAs for 16 rows; only bonds with a site inside test anything per row.
+// it touches) of the warp's list, and costs one address and, for 16 (8) rows, 4 (8) loads per
+// lane and their FMAs; only bonds with a site inside test anything per row.
 // Every row sums its terms in a fixed order: deterministic.
 //
 // What bounds it: FP32 L2-to-SM traffic (about 11 reads of 128 bytes per row and
@@ -45,7 +45,7 @@
 // by row, testing each bond on each row (74 to 80 warp instructions per row and
 // pass).  ms per cTPQ step (6 stages), before and now: 26 sites of a 3-regular
 // graph FP32 118.6 -> 103, 25-site chain FP32 50.7 -> 43.4, 21-site ladder FP64
-// 25.5 -> 21.5, 22 sites FP64 57 -> 44.  Tried (26 sites): 24 warps per SM 123, 32
+// 25.5 -> 14.2, 22 sites FP64 57 -> 29.5.  Tried (26 sites): 24 warps per SM 123, 32
 // 206 (more rows in flight leave L2 early), 2 rows per lane 122 to 217.
 #include "fixed.cuh"
 #include "hvcommon.cuh"
@@ -62,25 +62,30 @@ namespace {
 
 constexpr int kTileThreads = 256;
 constexpr int kTileItemBits = 5;  // smallest tile
-constexpr int kTileRowBits = 2;   // item bits held in registers
-constexpr int kTileRows = 1 << kTileRowBits;  // rows of a lane
 // sites of an FP32 item order's leading cluster: 2^7 rows are in a thread block at a
 // time (26 sites: 103 against 106 ms a step in ascending order; FP64, bound by its
-// pipe: 45.5 against 44.3, so ascending)
+// pipe, was 3 % slower with it, so ascending there)
 constexpr int kTileCluster = 8;
 constexpr int kTileSlack = 1;     // half tiles that a block may be ahead of the average
 constexpr int kTileWaits = 64;    // pacing polls at most
 constexpr int kTileMin = 2;       // thread blocks per SM
-constexpr int kTileUnroll = 3;    // list entries in flight (8 16-byte loads per lane)
+// list entries in flight (FP32 12 16-byte, FP64 16 8-byte loads per lane)
+template <typename T> constexpr int kTileUnroll = sizeof(T) == 4 ? 3 : 2;
 
-// Lane layout of a 32-column row: every lane moves 16 bytes (E columns), LPR
-// lanes per row, 2^QB rows per warp access, 2^IB rows per item.
+// Lane layout of a 32-column row: E columns per lane, LPR lanes per row, 2^QB rows
+// per warp access, 2^RB rows per lane, 2^IB rows per item.  FP32 lanes move 16
+// bytes.  FP64 rows take a whole warp, so that which rows a bond touches is the
+// same for all lanes and the FP64 pipe gets no FMA for the others (with two rows
+// per access, masked, pass 1 of a 21-site chain ran 11 FP64 operations per
+// element, 6.3 of them needed).
 template <typename T>
 struct TileShape {
-    static constexpr int E = 16 / (int)sizeof(T);
+    static constexpr int E = sizeof(T) == 4 ? 4 : 1;
     static constexpr int LPR = 32 / E;
-    static constexpr int QB = sizeof(T) == 4 ? 2 : 1;
-    static constexpr int IB = QB + kTileRowBits;
+    static constexpr int QB = sizeof(T) == 4 ? 2 : 0;
+    static constexpr int RB = sizeof(T) == 4 ? 2 : 3;
+    static constexpr int R = 1 << RB;
+    static constexpr int IB = QB + RB;
 };
 
 // One applicable bond of a warp's item.
@@ -89,7 +94,7 @@ struct alignas(16) TileHit;
 template <>
 struct alignas(16) TileHit<float> {
     int row;        // target of the item's first row
-    uint32_t mask;  // rows (bits 0-3) and lane groups (bits 4-7) it applies to
+    uint32_t mask;  // rows (bits 0-3) and lane groups (bits 4-7) it applies to; FP64: rows (bits 0-7)
     float c;
 };
 template <>
@@ -99,33 +104,29 @@ struct alignas(16) TileHit<double> {
     uint32_t mask;
 };
 
-__device__ __forceinline__ void ld16(const float *p, float (&v)[4]) {
+__device__ __forceinline__ void ldrow(const float *p, float (&v)[4]) {
     asm("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p));
 }
-__device__ __forceinline__ void ld16(const double *p, double (&v)[2]) {
-    asm("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "l"(p));
+__device__ __forceinline__ void ldrow(const double *p, double (&v)[1]) {
+    asm("ld.global.nc.f64 %0, [%1];" : "=d"(v[0]) : "l"(p));
 }
 // streamed rows (t, the old y and v, the stores), evicted from L2 first
-__device__ __forceinline__ void ldc16(const float *p, float (&v)[4], uint64_t pol) {  // coherent: may alias y
+__device__ __forceinline__ void ldrow_rw(const float *p, float (&v)[4], uint64_t pol) {  // coherent: may alias y
     asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
                  : "l"(p), "l"(pol)
                  : "memory");
 }
-__device__ __forceinline__ void ldc16(const double *p, double (&v)[2], uint64_t pol) {
-    asm volatile("ld.global.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;"
-                 : "=d"(v[0]), "=d"(v[1])
-                 : "l"(p), "l"(pol)
-                 : "memory");
+__device__ __forceinline__ void ldrow_rw(const double *p, double (&v)[1], uint64_t pol) {
+    asm volatile("ld.global.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v[0]) : "l"(p), "l"(pol) : "memory");
 }
-__device__ __forceinline__ void st16(float *p, const float (&v)[4], uint64_t pol) {
+__device__ __forceinline__ void strow(float *p, const float (&v)[4], uint64_t pol) {
     asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "f"(v[0]), "f"(v[1]),
                  "f"(v[2]), "f"(v[3]), "l"(pol)
                  : "memory");
 }
-__device__ __forceinline__ void st16(double *p, const double (&v)[2], uint64_t pol) {
-    asm volatile("st.global.L2::cache_hint.v2.f64 [%0], {%1, %2}, %3;" ::"l"(p), "d"(v[0]), "d"(v[1]), "l"(pol)
-                 : "memory");
+__device__ __forceinline__ void strow(double *p, const double (&v)[1], uint64_t pol) {
+    asm volatile("st.global.L2::cache_hint.f64 [%0], %1, %2;" ::"l"(p), "d"(v[0]), "l"(pol) : "memory");
 }
 
 template <typename T>
@@ -145,9 +146,20 @@ __device__ __forceinline__ void tile_fma(float c, const float (&v)[4], float (&a
     fma2(acc[0], acc[1], c, v[0], v[1]);
     fma2(acc[2], acc[3], c, v[2], v[3]);
 }
-__device__ __forceinline__ void tile_fma(double c, const double (&v)[2], double (&acc)[2]) {
+__device__ __forceinline__ void tile_fma(double c, const double (&v)[1], double (&acc)[1]) {
     acc[0] = fma(c, v[0], acc[0]);
-    acc[1] = fma(c, v[1], acc[1]);
+}
+
+// One bond on the rows of MASK only (FP64; no instruction for the other rows).
+template <uint32_t MASK>
+__device__ __forceinline__ void tile_some(const double *p, const int64_t (&roff)[8], double c, double (&acc)[8][1]) {
+    double v[8][1];
+#pragma unroll
+    for (int j = 0; j < 8; j++)
+        if ((MASK >> j) & 1u) ldrow(p + roff[j], v[j]);
+#pragma unroll
+    for (int j = 0; j < 8; j++)
+        if ((MASK >> j) & 1u) tile_fma(c, v[j], acc[j]);
 }
 
 // One pass.  PASS 1 writes t; PASS 2 reads t and applies the epilogue.
@@ -156,7 +168,8 @@ __global__ void __launch_bounds__(kTileThreads, kTileMin)
     k_tile(const __grid_constant__ HvArgs<T> a, const __grid_constant__ TileArgs ta, const T *__restrict__ diag,
            T *tbuf) {
     using S = TileShape<T>;
-    constexpr int E = S::E, LPR = S::LPR, QB = S::QB, IB = S::IB, R = kTileRows;
+    constexpr int E = S::E, LPR = S::LPR, QB = S::QB, IB = S::IB, RB = S::RB, R = S::R;
+    constexpr int UN = kTileUnroll<T>;
     constexpr int W = kTileThreads / 32, P = PASS - 1;
     constexpr int NR = RED == 2 ? 3 : (RED ? 1 : 0);
     __shared__ uint32_t pin[4][256], pout[4][256];
@@ -183,14 +196,19 @@ __global__ void __launch_bounds__(kTileThreads, kTileMin)
     const T *__restrict__ X = a.x;
     // row offsets of the item's rows: lane group, register rows; lane l also holds row
     // l of the item (group l mod 2^QB, register row l >> QB) for the diagonal
-    const int qoff = ((rsub & 1) ? ta.site[P][0] : 0) + (QB == 2 && (rsub & 2) ? ta.site[P][1] : 0);
-    const int r1 = ta.site[P][QB], r2 = kTileRowBits > 1 ? ta.site[P][QB + 1] : 0;
-    const int drow = ((lane & 1) ? ta.site[P][0] : 0) + (QB == 2 && (lane & 2) ? ta.site[P][1] : 0) +
-                     (((lane >> QB) & 1) ? r1 : 0) + (((lane >> QB) & 2) ? r2 : 0);
-    const int64_t el = (int64_t)qoff * 32 + E * gl;  // this lane's element of the item's first row
+    int drow = 0;
+#pragma unroll
+    for (int b = 0; b < IB; b++) drow += ((lane >> b) & 1) ? ta.site[P][b] : 0;
     int64_t roff[R];
 #pragma unroll
-    for (int j = 0; j < R; j++) roff[j] = el + (int64_t)((j & 1 ? r1 : 0) + (j & 2 ? r2 : 0)) * 32;
+    for (int j = 0; j < R; j++) {
+        int r = 0;
+#pragma unroll
+        for (int b = 0; b < QB; b++) r += ((rsub >> b) & 1) ? ta.site[P][b] : 0;
+#pragma unroll
+        for (int b = 0; b < RB; b++) r += ((j >> b) & 1) ? ta.site[P][QB + b] : 0;
+        roff[j] = (int64_t)r * 32 + E * gl;
+    }
     const bool use_beta = a.beta != 0.0, use_v = a.v != nullptr;
     const uint32_t lt = (1u << lane) - 1u;
     const uint64_t stream = spol(1, 1);
@@ -278,7 +296,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileMin)
         if constexpr (PASS == 1) {
             const T dv = lane < (1 << IB) ? __ldg(diag + (int64_t)s + drow) : (T)0;
 #pragma unroll
-            for (int j = 0; j < R; j++) ld16(X + base + roff[j], acc[j]);
+            for (int j = 0; j < R; j++) ldrow(X + base + roff[j], acc[j]);
 #pragma unroll
             for (int j = 0; j < R; j++) {
                 const T dj = __shfl_sync(0xffffffffu, dv, (j << QB) | rsub);
@@ -287,54 +305,77 @@ __global__ void __launch_bounds__(kTileThreads, kTileMin)
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < R; j++) ldc16(tbuf + base + roff[j], acc[j], stream);
+            for (int j = 0; j < R; j++) ldrow_rw(tbuf + base + roff[j], acc[j], stream);
         }
         int k = 0;
 #pragma unroll 1
-        for (; k + kTileUnroll <= nf; k += kTileUnroll) {
-            T v[kTileUnroll][R][E], c[kTileUnroll];
+        for (; k + UN <= nf; k += UN) {
+            T v[UN][R][E], c[UN];
 #pragma unroll
-            for (int u = 0; u < kTileUnroll; u++) {
+            for (int u = 0; u < UN; u++) {
                 const TileHit<T> h = hit[k + u];
                 c[u] = h.c;
                 const T *p = X + (int64_t)h.row * 32;
 #pragma unroll
-                for (int j = 0; j < R; j++) ld16(p + roff[j], v[u][j]);
+                for (int j = 0; j < R; j++) ldrow(p + roff[j], v[u][j]);
             }
 #pragma unroll
-            for (int u = 0; u < kTileUnroll; u++)
+            for (int u = 0; u < UN; u++)
 #pragma unroll
                 for (int j = 0; j < R; j++) tile_fma(c[u], v[u][j], acc[j]);
         }
-        // the rest: whole items left over and bonds with a site inside the item.  What
-        // is not loaded is 0 (FP64 skips the FMAs of rows it does not touch).
+        // the rest: whole items left over and bonds with a site inside the item
+        if constexpr (sizeof(T) == 8) {
 #pragma unroll 1
-        for (; k < nh; k += kTileUnroll) {
-            T v[kTileUnroll][R][E], c[kTileUnroll];
-            uint32_t rows[kTileUnroll];
-#pragma unroll
-            for (int u = 0; u < kTileUnroll; u++) {
-                const TileHit<T> h = hit[k + u < nh ? k + u : k];
-                c[u] = h.c;
-                rows[u] = k + u < nh ? h.mask & 0xFu : 0u;
-                const bool mine = (h.mask >> (4 + rsub)) & 1u;
+            for (; k < nh; k++) {
+                const TileHit<T> h = hit[k];
                 const T *p = X + (int64_t)h.row * 32;
-#pragma unroll
-                for (int j = 0; j < R; j++) {
-#pragma unroll
-                    for (int e = 0; e < E; e++) v[u][j][e] = (T)0;
-                    if (mine && ((rows[u] >> j) & 1u)) ld16(p + roff[j], v[u][j]);
+                switch (h.mask & 0xFFu) {  // by the values of one item bit, or of two that differ
+                case 0x55u: tile_some<0x55u>(p, roff, h.c, acc); break;
+                case 0xAAu: tile_some<0xAAu>(p, roff, h.c, acc); break;
+                case 0x33u: tile_some<0x33u>(p, roff, h.c, acc); break;
+                case 0xCCu: tile_some<0xCCu>(p, roff, h.c, acc); break;
+                case 0x0Fu: tile_some<0x0Fu>(p, roff, h.c, acc); break;
+                case 0xF0u: tile_some<0xF0u>(p, roff, h.c, acc); break;
+                case 0x22u: tile_some<0x22u>(p, roff, h.c, acc); break;
+                case 0x44u: tile_some<0x44u>(p, roff, h.c, acc); break;
+                case 0x0Au: tile_some<0x0Au>(p, roff, h.c, acc); break;
+                case 0x50u: tile_some<0x50u>(p, roff, h.c, acc); break;
+                case 0x0Cu: tile_some<0x0Cu>(p, roff, h.c, acc); break;
+                case 0x30u: tile_some<0x30u>(p, roff, h.c, acc); break;
+                default: tile_some<0xFFu>(p, roff, h.c, acc); break;
                 }
             }
+        } else {
+            // what is not loaded is 0
+#pragma unroll 1
+            for (; k < nh; k += UN) {
+                T v[UN][R][E], c[UN];
+                uint32_t rows[UN];
 #pragma unroll
-            for (int u = 0; u < kTileUnroll; u++)
+                for (int u = 0; u < UN; u++) {
+                    const TileHit<T> h = hit[k + u < nh ? k + u : k];
+                    c[u] = h.c;
+                    rows[u] = k + u < nh ? h.mask & 0xFu : 0u;
+                    const bool mine = (h.mask >> (4 + rsub)) & 1u;
+                    const T *p = X + (int64_t)h.row * 32;
 #pragma unroll
-                for (int j = 0; j < R; j++)
-                    if (sizeof(T) == 4 || ((rows[u] >> j) & 1u)) tile_fma(c[u], v[u][j], acc[j]);
+                    for (int j = 0; j < R; j++) {
+#pragma unroll
+                        for (int e = 0; e < E; e++) v[u][j][e] = (T)0;
+                        if (mine && ((rows[u] >> j) & 1u)) ldrow(p + roff[j], v[u][j]);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < UN; u++)
+#pragma unroll
+                    for (int j = 0; j < R; j++)
+                        tile_fma(c[u], v[u][j], acc[j]);
+            }
         }
         if constexpr (PASS == 1) {
 #pragma unroll
-            for (int j = 0; j < R; j++) st16(tbuf + base + roff[j], acc[j], stream);
+            for (int j = 0; j < R; j++) strow(tbuf + base + roff[j], acc[j], stream);
         } else {
             if constexpr (RED == 2) {
                 RedAcc<T> r[3][E];
@@ -343,7 +384,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileMin)
 #pragma unroll
                 for (int j = 0; j < R; j++) {
                     T xo[E];
-                    ld16(X + base + roff[j], xo);
+                    ldrow(X + base + roff[j], xo);
 #pragma unroll
                     for (int e = 0; e < E; e++) {
                         r[0][e].add(xo[e], acc[j][e]);
@@ -364,12 +405,19 @@ __global__ void __launch_bounds__(kTileThreads, kTileMin)
 #pragma unroll
             for (int j = 0; j < R; j++)
 #pragma unroll
-                for (int e = 0; e < E; e++) out[j][e] = al[e] * (a.swap ? acc[j][e ^ 1] : acc[j][e]);
+                for (int e = 0; e < E; e++) {
+                    T hx = acc[j][e];
+                    if (a.swap) {  // the partner column: in this lane, or in the next
+                        if constexpr (E == 1) hx = __shfl_xor_sync(0xffffffffu, hx, 1);
+                        else hx = acc[j][e ^ 1];
+                    }
+                    out[j][e] = al[e] * hx;
+                }
             if (use_beta) {
                 const T be = (T)a.beta;
                 T o[R][E];
 #pragma unroll
-                for (int j = 0; j < R; j++) ldc16(a.y + base + roff[j], o[j], stream);
+                for (int j = 0; j < R; j++) ldrow_rw(a.y + base + roff[j], o[j], stream);
 #pragma unroll
                 for (int j = 0; j < R; j++)
 #pragma unroll
@@ -378,14 +426,14 @@ __global__ void __launch_bounds__(kTileThreads, kTileMin)
             if (use_v) {
                 T o[R][E];
 #pragma unroll
-                for (int j = 0; j < R; j++) ldc16(a.v + base + roff[j], o[j], stream);
+                for (int j = 0; j < R; j++) ldrow_rw(a.v + base + roff[j], o[j], stream);
 #pragma unroll
                 for (int j = 0; j < R; j++)
 #pragma unroll
                     for (int e = 0; e < E; e++) out[j][e] = fma(ga[e], o[j][e], out[j][e]);
             }
 #pragma unroll
-            for (int j = 0; j < R; j++) st16(a.y + base + roff[j], out[j], stream);
+            for (int j = 0; j < R; j++) strow(a.y + base + roff[j], out[j], stream);
             if constexpr (RED == 1 || RED == 3) {
                 RedAcc<T> r[E];
 #pragma unroll
@@ -393,7 +441,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileMin)
 #pragma unroll
                 for (int j = 0; j < R; j++) {
                     T xo[E];
-                    if constexpr (RED == 1) ld16(X + base + roff[j], xo);
+                    if constexpr (RED == 1) ldrow(X + base + roff[j], xo);
 #pragma unroll
                     for (int e = 0; e < E; e++) r[e].add(RED == 1 ? xo[e] : out[j][e], out[j][e]);
                 }
@@ -611,27 +659,25 @@ int build_tile_tables(hphi_ctx *ctx, hphi_ham *H, int prec) {
         const std::vector<int> order = site_order(N, S[p], part[p], prec ? 0 : kTileCluster);
         // item bits: the first sites of that order (lane groups, then register rows)
         const int qb = prec ? TileShape<double>::QB : TileShape<float>::QB;
+        const int rb = prec ? TileShape<double>::RB : TileShape<float>::RB;
         int where[32];  // item bit of a site, -1: none
         for (int v = 0; v < 32; v++) where[v] = -1;
         int nitem = 0;
         for (int v : order)
-            if (nitem < qb + kTileRowBits) {
+            if (nitem < qb + rb) {
                 ta.site[p][nitem] = 1 << v;
                 where[v] = nitem++;
             }
-        // rows (bits 0-3) and lane groups (bits 4-7) whose item bit b has the value val
-        const uint32_t all_rows = 0xFu | ((1u << (1 << qb)) - 1u) << 4;
+        // rows (low bits) and lane groups (bits 4-7, FP32) whose item bit b has the value val
         auto rows_with = [&](int b, int val) {
             uint32_t m = 0;
-            if (b < qb) {
-                for (int g = 0; g < (1 << qb); g++)
-                    if (((g >> b) & 1) == val) m |= 1u << (4 + g);
-                return m | 0xFu;
-            }
-            for (int j = 0; j < kTileRows; j++)
-                if (((j >> (b - qb)) & 1) == val) m |= 1u << j;
-            return m | (all_rows & 0xF0u);
+            for (int j = 0; j < (1 << rb); j++)
+                if (b < qb || ((j >> (b - qb)) & 1) == val) m |= 1u << j;
+            for (int g = 0; qb > 0 && g < (1 << qb); g++)
+                if (b >= qb || ((g >> b) & 1) == val) m |= 1u << (4 + g);
+            return m;
         };
+        const uint32_t all_rows = 0xFFu;
         std::vector<TileEnt> full, rest;
         for (const TileBond &b : part[p]) {
             const int wi = where[b.i], wj = where[b.j];
