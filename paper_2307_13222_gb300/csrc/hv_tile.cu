@@ -30,15 +30,15 @@
 //
 // Inside a pass, a warp owns an item: the rows that share all bits but the
 // first item bits of S_k (16 rows in FP32, 4 per lane, 16 bytes of a row per lane;
-// 8 in FP64, all in every lane, one column per lane).  What a bond does to an item is decided once, one bond
-// per lane: with both sites outside the item it applies to all its rows or to
-// none; with one site inside, to the rows whose bit is the opposite of the other
-// site's; with both inside, to the rows where the two differ, in two parts.  In
-// every case the target rows lie at one fixed row offset, so an applicable bond
-// is an entry (first target row, coefficient, masks of the rows and lane groups
-// it touches) of the warp's list, and costs one address and, for 16 (8) rows, 4 (8) loads per
-// lane and their FMAs; only bonds with a site inside test anything per row.
-// Every row sums its terms in a fixed order: deterministic.
+// 8 in FP64, all in every lane, one column per lane).  What a bond does to an item
+// is decided once, one bond per lane: with both sites outside the item it applies
+// to all its rows or to none; with one site inside, to the rows whose bit is the
+// opposite of the other site's; with both inside, to the rows where the two
+// differ, in two parts.  In every case the target rows lie at one fixed row
+// offset, so an applicable bond is an entry (first target row, coefficient, masks
+// of the rows and lane groups it touches) of the warp's list, and costs one address
+// and, for 16 (8) rows, 4 (8) loads per lane and their FMAs; only bonds with a site
+// inside test anything per row.  Every row sums its terms in a fixed order: deterministic.
 //
 // What bounds it: FP32 L2-to-SM traffic (about 11 reads of 128 bytes per row and
 // pass, 9 to 10 TB/s), FP64 the FP64 pipe.  Before, 8 lanes walked the bonds row
@@ -548,7 +548,19 @@ bool find_cover(int N, const std::vector<uint64_t> &adj, int smax, uint64_t *A_o
     };
     for (int st = 0; st < N; st++) {
         uint64_t A = 1ull << st;
-        while (__builtin_popcountll(A) < need) {
+        while (true) {
+            const uint64_t R = all & ~(A | nbr(A));
+            if (__builtin_popcountll(A) >= need && __builtin_popcountll(R) >= need) {
+                // B: `need` sites of R (the fewest that bring pass 2 within smax;
+                // the sites left out keep their bonds free for either pass)
+                uint64_t B = 0;
+                for (int v = 0; v < N && __builtin_popcountll(B) < need; v++)
+                    if ((R >> v) & 1) B |= 1ull << v;
+                *A_out = A;
+                *B_out = B;
+                return true;
+            }
+            if (__builtin_popcountll(A) >= need) break;
             const uint64_t cand = nbr(A) ? nbr(A) : (all & ~A);
             int best = -1, bc = 1 << 30;
             for (int v = 0; v < N; v++) {
@@ -561,17 +573,6 @@ bool find_cover(int N, const std::vector<uint64_t> &adj, int smax, uint64_t *A_o
             }
             if (best < 0) break;
             A |= 1ull << best;
-            const uint64_t R = all & ~(A | nbr(A));
-            if (__builtin_popcountll(A) >= need && __builtin_popcountll(R) >= need) {
-                // B: `need` sites of R (the fewest that bring pass 2 within smax;
-                // the sites left out keep their bonds free for either pass)
-                uint64_t B = 0;
-                for (int v = 0; v < N && __builtin_popcountll(B) < need; v++)
-                    if ((R >> v) & 1) B |= 1ull << v;
-                *A_out = A;
-                *B_out = B;
-                return true;
-            }
         }
     }
     return false;
