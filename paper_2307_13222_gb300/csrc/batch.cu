@@ -520,6 +520,16 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
         P.y = P.scal + 2;
         P.state = iws + 2 * p;
     }
+    // launch order: long problems first, so that none starts when the others are done (200
+    // chains of 12 to 16 sites, one block each on 152 SMs)
+    std::vector<int> order(nprob);
+    for (int p = 0; p < nprob; p++) order[p] = p;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return hams[x]->D > hams[y]->D; });
+    std::vector<BProb> lp(nprob);  // descriptors in that order
+    auto send = [&]() {
+        for (int q = 0; q < nprob; q++) lp[q] = hp[order[q]];
+        return cudaMemcpyAsync(dprob, lp.data(), sizeof(BProb) * nprob, cudaMemcpyHostToDevice, ctx->stream);
+    };
     HPHI_CUDA(ctx, cudaMemsetAsync(iws, 0, 2 * (size_t)nprob * sizeof(int), ctx->stream));
     // host mirrors of alpha / beta^2 (step-major) and the stopping state
     std::vector<double> ah((size_t)M * nprob, 0.0), b2h((size_t)(M + 1) * nprob, 0.0);
@@ -578,16 +588,23 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
         }
     };
     const int nthreads = nprob >= 64 ? std::max(1, std::min(16, (int)std::thread::hardware_concurrency())) : 1;
+    // Large batches run one chunk ahead of the checks: the tridiagonal problems of 200 small
+    // solves take the host longer than 8 steps take the GPU (a problem that turns out to be
+    // finished ignores its extra steps).  Small batches wait for the check instead.
+    const bool ahead = nthreads > 1;
+    auto launch = [&](int k0) -> int {
+        for (int p = 0; p < nprob; p++) {
+            hp[p].k0 = k0;
+            hp[p].nsteps = done[p] ? 0 : std::min(chunk, M - k0);
+        }
+        HPHI_CUDA(ctx, send());
+        return batch_launch_steps(ctx, dprob, nprob, dyn_bytes);
+    };
     int k = 0, left = nprob;
+    int stl = launch(0);
+    if (stl) return fail(stl);
     while (left > 0 && k < M) {
         const int c = std::min(chunk, M - k);
-        for (int p = 0; p < nprob; p++) {
-            hp[p].k0 = k;
-            hp[p].nsteps = done[p] ? 0 : c;
-        }
-        HPHI_CUDA(ctx, cudaMemcpyAsync(dprob, hp.data(), sizeof(BProb) * nprob, cudaMemcpyHostToDevice, ctx->stream));
-        int stl = batch_launch_steps(ctx, dprob, nprob, dyn_bytes);
-        if (stl) return fail(stl);
         HPHI_CUDA(ctx, cudaMemcpyAsync(ist.data(), iws, sizeof(int) * 2 * nprob, cudaMemcpyDeviceToHost, ctx->stream));
         HPHI_CUDA(ctx, cudaMemcpyAsync(ah.data() + (size_t)k * nprob, alpha_all + (size_t)k * nprob,
                                        sizeof(double) * (size_t)c * nprob, cudaMemcpyDeviceToHost, ctx->stream));
@@ -598,6 +615,7 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
         HPHI_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         const int k_prev = k;
         k += c;
+        if (ahead && k < M && (stl = launch(k))) return fail(stl);
         if (nthreads == 1) {
             std::vector<double> ap, bp;
             for (int p = 0; p < nprob; p++)
@@ -614,6 +632,7 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
         }
         left = 0;
         for (int p = 0; p < nprob; p++) left += !done[p];
+        if (!ahead && left > 0 && k < M && (stl = launch(k))) return fail(stl);
     }
     // energies (eigenvalues of T_m) and, where asked for, the Ritz vector of T_m
     // for the ground-state pass; spread over host threads for large batches
@@ -626,18 +645,16 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
         const int m = mstop[p];
         if (st[p] || m < 1) return;
         const bool want = gs_out && gs_out[p];
-        std::vector<double> a(m), bb(m, 0.0), ev(m), Z(want ? (size_t)m * m : 0);
+        std::vector<double> a(m), b2(m + 1);
         for (int j = 0; j < m; j++) a[j] = ah[(size_t)j * nprob + p];
-        for (int j = 1; j < m; j++) bb[j] = sqrt(b2h[(size_t)j * nprob + p]);
-        int s2 = hphi_tridiag_eigen(m, a.data(), bb.data(), ev.data(), want ? Z.data() : nullptr);
+        for (int j = 0; j <= m; j++) b2[j] = b2h[(size_t)j * nprob + p];
+        std::vector<double> y;
+        const int s2 = lowest_vector(m, a.data(), b2.data(), &theta[p], y);
         if (s2) {
             st[p] = s2;
             return;
         }
-        theta[p] = ev[0];
-        if (!want) return;
-        yv[p].resize(m);
-        for (int i = 0; i < m; i++) yv[p][i] = Z[(size_t)i * m];
+        if (want) yv[p].swap(y);
     };
     if (nthreads == 1) {
         for (int p = 0; p < nprob; p++) finish(p);
@@ -649,11 +666,13 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
             });
         for (auto &th : pool) th.join();
     }
+    // the Ritz vectors in one copy (with the per-problem scalars, which are spent by now)
+    std::vector<double> yall;
     for (int p = 0; p < nprob; p++) {
         if (yv[p].empty()) continue;
+        if (yall.empty()) yall.assign(n_pp, 0.0);
         const int m = (int)yv[p].size();
-        HPHI_CUDA(ctx, cudaMemcpyAsync((double *)hp[p].y, yv[p].data(), sizeof(double) * m, cudaMemcpyHostToDevice,
-                                       ctx->stream));
+        std::copy(yv[p].begin(), yv[p].end(), yall.begin() + (size_t)p * (M + 2) + 2);
         hp[p].m = m;
         hp[p].theta = theta[p];
         hp[p].gs = (double *)gs_out[p];
@@ -661,7 +680,8 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
     }
     std::vector<double> gres(nprob, -1.0);
     if (any_gs) {
-        HPHI_CUDA(ctx, cudaMemcpyAsync(dprob, hp.data(), sizeof(BProb) * nprob, cudaMemcpyHostToDevice, ctx->stream));
+        HPHI_CUDA(ctx, cudaMemcpyAsync(pp, yall.data(), sizeof(double) * n_pp, cudaMemcpyHostToDevice, ctx->stream));
+        HPHI_CUDA(ctx, send());
         int stg = batch_launch_gs(ctx, dprob, nprob, dyn_bytes);
         if (stg) return fail(stg);
         std::vector<double> pph(n_pp);

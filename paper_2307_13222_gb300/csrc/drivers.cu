@@ -151,7 +151,8 @@ static int sturm_below(int n, const double *a, const double *b, double x, double
 // lowest eigenvalue, otherwise (or without a warm start) bisection on the
 // Sturm count decides.  *warm receives the result.  The full eigenvector is
 // formed only at the end of a run.
-int lowest_ritz_warm(int m, const double *alpha, const double *beta2, double *warm, double *theta, double *ylast) {
+int lowest_ritz_warm(int m, const double *alpha, const double *beta2, double *warm, double *theta, double *ylast,
+                     std::vector<double> *vec) {
     std::vector<double> b(m + 1, 0.0), y(m);
     double lo = alpha[0], scale = 0.0;
     for (int j = 1; j < m; j++) b[j] = sqrt(beta2[j]);
@@ -217,6 +218,33 @@ int lowest_ritz_warm(int m, const double *alpha, const double *beta2, double *wa
     *theta = t;
     *ylast = fabs(y[m - 1]);
     if (warm) *warm = t;
+    if (vec) {
+        // the eigenvector (first component non-negative) and its Rayleigh quotient, if
+        // the second eigenvalue is not a near copy of the first; empty otherwise
+        vec->clear();
+        if (m > 1 && sturm_below(m, alpha, b.data(), t + 1e-8 * scale, tiny) != 1) return HPHI_OK;
+        *theta = rayleigh();
+        if (y[0] < 0.0)
+            for (int j = 0; j < m; j++) y[j] = -y[j];
+        vec->swap(y);
+    }
+    return HPHI_OK;
+}
+
+// Lowest eigenvalue and eigenvector of T_m in O(m) steps (inverse iteration);
+// where the two lowest eigenvalues are too close for it, from the full QL
+// eigensystem.  (QL forms all m vectors, O(m^3) on the host: 1 to 2 ms at m = 80, 15
+// of the 28 ms of a batch of 200.)
+int lowest_vector(int m, const double *alpha, const double *beta2, double *theta, std::vector<double> &y) {
+    double yl = 0.0;
+    int st = lowest_ritz_warm(m, alpha, beta2, nullptr, theta, &yl, &y);
+    if (st || !y.empty()) return st;
+    std::vector<double> b(m, 0.0), ev(m), Z((size_t)m * m);
+    for (int j = 1; j < m; j++) b[j] = sqrt(beta2[j]);
+    if ((st = hphi_tridiag_eigen(m, alpha, b.data(), ev.data(), Z.data()))) return st;
+    *theta = ev[0];
+    y.assign(m, 0.0);
+    for (int i = 0; i < m; i++) y[i] = Z[(size_t)i * m];
     return HPHI_OK;
 }
 
@@ -516,12 +544,9 @@ static int lanczos_reorth(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lanczos
         for (int j = 0; j <= M; j++) beta_host[j] = (j >= 1 && j <= m) ? sqrt(beta2_h[j]) : 0.0;
     if (gs_out) {
         {
-            std::vector<double> a(alpha_h.begin(), alpha_h.begin() + m), b(m, 0.0), ev(m), Z((size_t)m * m);
-            for (int j = 1; j < m; j++) b[j] = sqrt(beta2_h[j]);
-            if ((st = hphi_tridiag_eigen(m, a.data(), b.data(), ev.data(), Z.data())))
+            double t0 = 0.0;
+            if ((st = lowest_vector(m, alpha_h.data(), beta2_h.data(), &t0, y)))
                 return fail(set_err(ctx, st, "tridiagonal eigensolver failed"));
-            y.assign(m, 0.0);
-            for (int i = 0; i < m; i++) y[i] = Z[(size_t)i * m];
         }
         // x = sum_j y_j v_j, as gs -= sum_j (-y_j) v_j from zero
         std::vector<double> ny(m);
@@ -612,16 +637,7 @@ extern "C" int hphi_lanczos(hphi_ctx *ctx, const hphi_ham *ham, const hphi_lancz
         return HPHI_OK;
     };
     // the Ritz vector of T_m (for the ground-state pass)
-    auto full_y = [&](int m) -> int {
-        std::vector<double> a(alpha_h.begin(), alpha_h.begin() + m), b(m, 0.0), ev(m), Z((size_t)m * m);
-        for (int j = 1; j < m; j++) b[j] = sqrt(beta2_h[j]);
-        int s2 = hphi_tridiag_eigen(m, a.data(), b.data(), ev.data(), Z.data());
-        if (s2) return s2;
-        theta = ev[0];
-        y.assign(m, 0.0);
-        for (int i = 0; i < m; i++) y[i] = Z[(size_t)i * m];
-        return HPHI_OK;
-    };
+    auto full_y = [&](int m) -> int { return lowest_vector(m, alpha_h.data(), beta2_h.data(), &theta, y); };
 
     for (int k = 0; k < M; k++) {
         HvLaunch A{};

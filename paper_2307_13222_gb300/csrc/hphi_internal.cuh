@@ -375,7 +375,10 @@ int tridiag_ql(int n, double *d, double *e, double *z);
 // and |last component| of its normalised eigenvector
 int lowest_ritz(int m, const double *alpha, const double *beta2, double *theta, double *ylast);
 // the same with a warm start (an upper bound of the lowest eigenvalue, updated)
-int lowest_ritz_warm(int m, const double *alpha, const double *beta2, double *warm, double *theta, double *ylast);
+int lowest_ritz_warm(int m, const double *alpha, const double *beta2, double *warm, double *theta, double *ylast,
+                     std::vector<double> *vec = nullptr);
+// lowest eigenvalue and its eigenvector (first component non-negative)
+int lowest_vector(int m, const double *alpha, const double *beta2, double *theta, std::vector<double> &y);
 
 // ---- high-high pass table (hv_seg.cu) ------------------------------------------------
 int build_seg_tables(hphi_ctx *ctx, hphi_ham *H);
