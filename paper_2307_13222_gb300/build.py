@@ -44,8 +44,9 @@ def _stale() -> bool:
 # the basis / Hamiltonian table builders
 HV_COMMON = ["basis.cu", "ham.cu", "hvcommon.cuh", "rowvisit.cuh", "hphi_internal.cuh"]
 # units that name kernels defined in other files (hv.cu launches the lean and
-# the on-the-fly kernels)
-TAG_DEPS = {"hv.cu": ["hv_lean.cu", "hv_fly.cu"]}
+# the on-the-fly kernels) or share a header of their own
+TAG_DEPS = {"hv.cu": ["hv_lean.cu", "hv_fly.cu"], "hv_warp.cu": ["fixed.cuh"], "hv_hub.cu": ["fixed.cuh"],
+            "hv_tile.cu": ["fixed.cuh"]}
 
 
 def source_tag(unit: str = "hv.cu") -> str:
