@@ -199,7 +199,8 @@ extern "C" int hphi_ctx_create(int device, void *stream, hphi_ctx **out) {
     c->stream = (cudaStream_t)stream;
     if (cudaSetDevice(device) != cudaSuccess ||
         cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-        ensure_dscal(c, 4096) != HPHI_OK || cudaMalloc(&c->dflag, sizeof(int)) != cudaSuccess) {
+        ensure_dscal(c, 4096) != HPHI_OK || cudaMalloc(&c->dflag, sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&c->ticket, 2 * sizeof(unsigned)) != cudaSuccess) {
         cudaGetLastError();
         hphi_ctx_destroy(c);
         return HPHI_E_CUDA;
