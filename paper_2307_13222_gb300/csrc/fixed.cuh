@@ -2,21 +2,31 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 
 namespace hphi {
 
-constexpr int kFixShift = 29;  // 64-bit to 32-bit fixed point (diagonals are below 2^59 in 64 bits)
-
+// A diagonal is an integer times a power of two, below 2^BITS in 64 bits; 32-bit
+// integers keep its upper bits (rounded), below 2^30.
 template <typename T>
 struct FixInt { using type = int; };
 template <>
 struct FixInt<double> { using type = long long; };
 
-// A 64-bit fixed-point value in T's fixed point (FP32: its upper bits, rounded).
-template <typename T>
-__host__ __device__ __forceinline__ typename FixInt<T>::type to_fix(long long v) {
-    if constexpr (sizeof(T) == 4) return (int)((v + (1ll << (kFixShift - 1))) >> kFixShift);
+// A 64-bit fixed-point value as an integer of type I.
+template <typename I, int BITS>
+__host__ __device__ __forceinline__ I to_fix(long long v) {
+    constexpr int S = BITS - 30;
+    if constexpr (sizeof(I) == 4) return (int)((long long)((unsigned long long)v + (1ull << (S - 1))) >> S);
     else return v;
+}
+
+// Does coupling v survive on the grid of `bits` bits below 2^e2 as it would in a
+// floating-point number of `digits` digits: on the grid exactly, or with that many
+// bits of it (an error of half a grid step is then no more than half an ulp)?
+inline bool fix_keeps(double v, int e2, int bits, int digits) {
+    const double f = fabs(ldexp(v, bits - e2));
+    return f >= ldexp(1.0, digits - 1) || f == rint(f);
 }
 
 // (a0, a1) += c (v0, v1), each rounded as a single fma

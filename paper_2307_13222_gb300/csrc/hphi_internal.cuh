@@ -141,13 +141,18 @@ struct HubV {        // V n_i n_j
     int i, j;
     long long v;
 };
-struct HubArgs {
-    int N, up_pad, ngrp, nv;      // up_pad: most up hops of a string, padded to 8
-    uint32_t nh, ddn;             // up and down strings
-    double scale64, scale32;      // fixed point to value
+struct HubFix {
+    int bytes;                    // integers that hold it: 8, 4 (the upper bits), 0 (no kernel)
+    int parts;                    // 2: V has a grid of its own (FP64)
+    double scale, vscale;         // fixed point to value; of that V
     const long long *ufix;        // device [32]: U per site
     const HubV *vfix;             // device [nv]
     const long long *dup, *ddnf;  // device: V terms of one species alone, per up / down string (null: none)
+};
+struct HubArgs {
+    int N, up_pad, ngrp, nv;      // up_pad: most up hops of a string, padded to 8
+    uint32_t nh, ddn;             // up and down strings
+    HubFix fix[2];                // FP32 vectors, FP64 vectors
 };
 
 // Lin tables of one species (spin string, or up / down fermion string).

@@ -321,9 +321,10 @@ int launch_typed(hphi_ctx *ctx, const hphi_ham *ham, HvLaunch &L) {
         const bool warp = ham->tune_variant < 0 && ham->warp && one_col &&
                           (std::is_same<T, double>::value ? ham->nlo < 16 : ham->D >= 16384);
         // Hubbard: one column or one aligned pair of columns (a complex vector), automatic where
-        // its tables exist (4x4 FP32 5.7 -> 3.4 ms, 6x2 complex FP64 0.149 -> 0.108 ms; 8 sites
+        // its tables exist for the vectors' type (4x4 FP32 5.7 -> 3.4 ms, 6x2 complex FP64 0.149 -> 0.108 ms; 8 sites
         // 10 us either way)
-        const bool hub = ham->tune_variant < 0 && ham->hub && same_ld && red_mode >= 0 && L.ldx == L.ncol &&
+        const bool hub = ham->tune_variant < 0 && ham->hub && ham->hub->fix[sizeof(T) == 8].bytes && same_ld &&
+                         red_mode >= 0 && L.ldx == L.ncol &&
                          (L.ncol == 1 ? !L.swap
                                       : L.ncol == 2 && aligned(xs, 2 * sizeof(T)) && aligned(ys, 2 * sizeof(T)) &&
                                             aligned(vs, 2 * sizeof(T)));

@@ -11,8 +11,12 @@
 //     row block u' and one FMA per value.
 // So the sums stay in registers and the list entries are read once per 16 bytes
 // of result.  The diagonal sum_i U_i n_iu n_id + sum V n_i n_j is summed in fixed
-// point (integers below 2^30, FP64 data 2^59): per up string, tables over groups
-// of 6 sites of dn.
+// point: per up string, tables over groups of 6 sites of dn.  The grid follows the
+// sum of the couplings' magnitudes, and a row without a doubly occupied site has no
+// U in it, so the integers are chosen by what the grid does to the smallest coupling
+// (build_hub_tables): FP32 vectors take 32 bits where every coupling keeps its 24,
+// else 64; FP64 vectors one grid or two, one for U and one for V, and the kernel
+// only where these cost less than the hops round.
 //
 // What bounds it: FP64 the FP64 pipe (88 % busy; a warp's down hops run as many
 // rounds as its longest list), FP32 the latency of the up-hop loads and the bank
@@ -39,6 +43,7 @@ namespace hphi {
 namespace {
 
 constexpr int kHubGroup = 6;  // sites per diagonal table
+constexpr int kHubBits = 62;  // the diagonal lies below 2^62 grid steps
 
 template <typename T>
 struct alignas(16) HubPack {
@@ -46,7 +51,7 @@ struct alignas(16) HubPack {
 };
 
 template <typename I, int U>
-struct alignas(sizeof(I) * U) IntPack {  // the diagonal parts of U up strings
+struct alignas(sizeof(I) * U < 16 ? sizeof(I) * U : 16) IntPack {  // the diagonal parts of U up strings
     I e[U];
 };
 
@@ -92,6 +97,10 @@ __device__ __forceinline__ void hub_store(T *y, uint32_t r, const T (&v)[C]) {
     else *(reinterpret_cast<double2 *>(y) + r) = make_double2(v[0], v[1]);
 }
 
+// Sums that a diagonal is made of: 2 where V has a grid of its own.
+template <typename T>
+__host__ __device__ __forceinline__ int hub_parts(const HubArgs &g) { return sizeof(T) == 8 ? g.fix[1].parts : 1; }
+
 // acc[i] += c v[i] over one pack
 __device__ __forceinline__ void pack_fma(float c, const HubPack<float> &v, float (&acc)[4]) {
 #pragma unroll
@@ -102,10 +111,9 @@ __device__ __forceinline__ void pack_fma(double c, const HubPack<double> &v, dou
     acc[1] = fma(c, v.e[1], acc[1]);
 }
 
-template <typename T, int C, int RED, int NT, int MINB>
+template <typename T, typename I, int C, int RED, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
     k_hub(const __grid_constant__ HvArgs<T> a, const __grid_constant__ HubArgs g) {
-    using I = typename FixInt<T>::type;
     constexpr int P = 16 / (int)sizeof(T), U = P / C;
     // dn strings of a thread at a time (an FP64 pair fills the pipe with one)
     constexpr int QB = sizeof(T) == 8 && C == 2 ? 1 : 2;
@@ -116,8 +124,10 @@ __global__ void __launch_bounds__(NT, MINB)
     HubPack<T> *xs = (HubPack<T> *)s_raw;
     HubHop<T> *hops = (HubHop<T> *)(xs + ddn);              // [U][up_pad], zeros behind the list
     I *tab = (I *)(hops + U * g.up_pad);                    // [ngrp][64][U]
-    I *wj = tab + U * g.ngrp * 64;                          // [U][32]
-    T *coef = (T *)(wj + U * 32);                           // [n_coef]
+    const HubFix &fx = g.fix[sizeof(T) == 8];
+    const int parts = hub_parts<T>(g);                      // sums of a diagonal: U and V apart, or together
+    I *wj = tab + parts * U * g.ngrp * 64;                  // [U][32]; a second set of both for V
+    T *coef = (T *)(wj + parts * U * 32);                   // [n_coef]
     __shared__ int nup[U];
     __shared__ I du[U];
     const HamDesc &D = *a.P.desc;
@@ -130,7 +140,7 @@ __global__ void __launch_bounds__(NT, MINB)
         ga[c] = (T)(a.gamma_dev ? a.gamma_dev[c] : a.gamma[c]);
     }
     const T fold = FOLD ? al[0] : (T)1;
-    const T dscale = (T)(sizeof(T) == 4 ? g.scale32 : g.scale64) * fold;
+    const T dscale = (T)fx.scale * fold, vscale = (T)fx.vscale * fold;
     for (int i = threadIdx.x; i < D.n_ncoef; i += NT) coef[i] = (T)D.coef[i] * fold;
     const T be = (T)a.beta;
     const bool use_beta = a.beta != 0.0, use_v = a.v != nullptr;
@@ -157,20 +167,21 @@ __global__ void __launch_bounds__(NT, MINB)
         for (int i = threadIdx.x; i < U * 32; i += NT) {
             const int u = i >> 5, j = i & 31;
             const uint32_t h = u0 + u;
-            I w = 0;
+            I w = 0, wv = 0;
             if (h < g.nh && j < g.N) {
                 const uint32_t su = a.P.states_up[h];
-                if ((su >> j) & 1u) w += to_fix<T>(g.ufix[j]);
+                if ((su >> j) & 1u) w += to_fix<I, kHubBits>(fx.ufix[j]);
                 for (int k = 0; k < g.nv; k++) {
-                    const HubV v = g.vfix[k];
-                    if (v.j == j && ((su >> v.i) & 1u)) w += to_fix<T>(v.v);
-                    if (v.i == j && ((su >> v.j) & 1u)) w += to_fix<T>(v.v);
+                    const HubV v = fx.vfix[k];
+                    if (v.j == j && ((su >> v.i) & 1u)) wv += to_fix<I, kHubBits>(v.v);
+                    if (v.i == j && ((su >> v.j) & 1u)) wv += to_fix<I, kHubBits>(v.v);
                 }
             }
-            wj[i] = w;
+            wj[i] = parts == 2 ? w : w + wv;
+            if (parts == 2) wj[U * 32 + i] = wv;
             if (j == 0) {
                 nup[u] = h < g.nh ? a.P.up_cnt[h] : 0;
-                du[u] = h < g.nh && g.dup ? to_fix<T>(g.dup[h]) : (I)0;
+                du[u] = h < g.nh && fx.dup ? to_fix<I, kHubBits>(fx.dup[h]) : (I)0;
             }
         }
         for (uint32_t q = threadIdx.x; q < ddn; q += NT) {
@@ -187,12 +198,13 @@ __global__ void __launch_bounds__(NT, MINB)
             xs[q] = x;
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < U * g.ngrp * 64; i += NT) {
-            const int u = i % U, r = i / U, gr = r >> 6;
+        for (int i = threadIdx.x; i < parts * U * g.ngrp * 64; i += NT) {
+            const int u = i % U, r = i / U, gr = r >> 6, v = parts == 2 && gr >= g.ngrp;
+            const int j0 = (gr - (v ? g.ngrp : 0)) * kHubGroup;
             I s = 0;
 #pragma unroll
             for (int k = 0; k < kHubGroup; k++)
-                if ((r >> k) & 1) s += wj[u * 32 + (gr * kHubGroup + k < 32 ? gr * kHubGroup + k : 31)];
+                if ((r >> k) & 1) s += wj[(v * U + u) * 32 + (j0 + k < 32 ? j0 + k : 31)];
             tab[i] = s;
         }
         __syncthreads();
@@ -207,19 +219,38 @@ __global__ void __launch_bounds__(NT, MINB)
                 q[b] = on[b] ? q0 + b * NT : q0;
                 const uint32_t s = __ldg(a.P.states_dn + q[b]);
                 cnt[b] = on[b] ? __ldg(a.P.ll_cnt + q[b]) : 0;
-                const I dl = g.ddnf ? to_fix<T>(__ldg(g.ddnf + q[b])) : (I)0;
+                const I dl = fx.ddnf ? to_fix<I, kHubBits>(__ldg(fx.ddnf + q[b])) : (I)0;
                 const HubPack<T> x = xs[q[b]];
+                // sum of one set of tables, on top of d
+                auto add = [&](const I *tb, I (&d)[U]) {
+                    for (int k = 0; k < g.ngrp; k++) {
+                        const IntPack<I, U> t = *(const IntPack<I, U> *)(tb + (k * 64 + ((s >> (kHubGroup * k)) & 63u)) * U);
+#pragma unroll
+                        for (int u = 0; u < U; u++) d[u] += t.e[u];
+                    }
+                };
                 I d[U];
 #pragma unroll
                 for (int u = 0; u < U; u++) d[u] = dl + du[u];
-                for (int k = 0; k < g.ngrp; k++) {
-                    const IntPack<I, U> t = *(const IntPack<I, U> *)(tab + (k * 64 + ((s >> (kHubGroup * k)) & 63u)) * U);
+                T dv[U];  // the V part, where it is summed apart
+                if constexpr (sizeof(T) == 8) {
 #pragma unroll
-                    for (int u = 0; u < U; u++) d[u] += t.e[u];
+                    for (int u = 0; u < U; u++) dv[u] = (T)0;
+                    if (parts == 2) {
+                        add(tab + U * g.ngrp * 64, d);
+#pragma unroll
+                        for (int u = 0; u < U; u++) {
+                            dv[u] = (T)d[u] * vscale;
+                            d[u] = 0;
+                        }
+                    }
                 }
+                add(tab, d);
 #pragma unroll
                 for (int u = 0; u < U; u++) {
-                    const T dt = (T)d[u] * dscale;
+                    T dt;
+                    if constexpr (sizeof(T) == 8) dt = fma((T)d[u], dscale, dv[u]);
+                    else dt = (T)d[u] * dscale;
 #pragma unroll
                     for (int c = 0; c < C; c++) acc[b][u * C + c] = dt * x.e[u * C + c];
                 }
@@ -361,44 +392,45 @@ __global__ void __launch_bounds__(NT, MINB)
 }
 
 template <typename T, int C>
-size_t hub_smem(const HubArgs &g, int ncoef) {
-    const size_t U = 16 / sizeof(T) / C, I = sizeof(typename FixInt<T>::type);
-    return (size_t)g.ddn * 16 + U * g.up_pad * sizeof(HubHop<T>) + U * (g.ngrp * 64 + 32) * I +
-           ncoef * sizeof(T);
+size_t hub_smem(const HubArgs &g, int ncoef, int int_bytes) {
+    const size_t U = 16 / sizeof(T) / C;
+    return (size_t)g.ddn * 16 + U * g.up_pad * sizeof(HubHop<T>) +
+           hub_parts<T>(g) * U * (g.ngrp * 64 + 32) * (size_t)int_bytes + ncoef * sizeof(T);
 }
 
-template <typename T, int C, int RED, int NT, int MINB>
+template <typename T, typename I, int C, int RED, int NT, int MINB>
 int go_hub(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int *grid) {
     const HubArgs &g = *ham->hub;
-    const size_t dyn = hub_smem<T, C>(g, ham->host.n_ncoef);
-    const int occ = dyn_occupancy(ctx, (const void *)k_hub<T, C, RED, NT, MINB>, NT, dyn);
+    const size_t dyn = hub_smem<T, C>(g, ham->host.n_ncoef, (int)sizeof(I));
+    const int occ = dyn_occupancy(ctx, (const void *)k_hub<T, I, C, RED, NT, MINB>, NT, dyn);
     if (occ < 1) return set_err(ctx, HPHI_E_INVAL, "Hubbard H*x: the rows of an up string do not fit in shared memory");
     constexpr int U = 16 / (int)sizeof(T) / C;
     // no more thread blocks than the partials of an H*x launch hold (8 per SM)
     const int64_t gr = std::min<int64_t>((int64_t)std::min(occ, 8) * ctx->sm_count, (g.nh + U - 1) / U);
     *grid = (int)(gr < 1 ? 1 : gr);
     const int slot = prof_begin(ctx, PROF_HV);
-    k_hub<T, C, RED, NT, MINB><<<*grid, NT, dyn, ctx->stream>>>(a, g);
-    snprintf(ctx->last_kernel, sizeof ctx->last_kernel, "k_hub<%s,C%d,%d,RED%d>@" HPHI_SRC_TAG, tname<T>(), C, NT, RED);
+    k_hub<T, I, C, RED, NT, MINB><<<*grid, NT, dyn, ctx->stream>>>(a, g);
+    snprintf(ctx->last_kernel, sizeof ctx->last_kernel, "k_hub<%s,C%d,%d,I%d,RED%d>@" HPHI_SRC_TAG, tname<T>(), C, NT,
+             (int)sizeof(I) * 8, RED);
     prof_end(ctx, slot);
     HPHI_CUDA(ctx, cudaGetLastError());
     return HPHI_OK;
 }
 
-template <typename T, int C, int RED>
+template <typename T, typename I, int C, int RED>
 int go_hub_size(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int *grid) {
-    if (ham->hub->ddn > 4096) return go_hub<T, C, RED, 1024, 1>(ctx, ham, a, grid);
-    if (ham->hub->ddn > 512) return go_hub<T, C, RED, 256, 4>(ctx, ham, a, grid);
-    return go_hub<T, C, RED, 64, 8>(ctx, ham, a, grid);
+    if (ham->hub->ddn > 4096) return go_hub<T, I, C, RED, 1024, 1>(ctx, ham, a, grid);
+    if (ham->hub->ddn > 512) return go_hub<T, I, C, RED, 256, 4>(ctx, ham, a, grid);
+    return go_hub<T, I, C, RED, 64, 8>(ctx, ham, a, grid);
 }
 
-template <typename T, int C>
+template <typename T, typename I, int C>
 int go_hub_red(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int red_mode, int *grid) {
     switch (red_mode) {
-    case 0: return go_hub_size<T, C, 0>(ctx, ham, a, grid);
-    case 1: return go_hub_size<T, C, 1>(ctx, ham, a, grid);
-    case 2: return go_hub_size<T, C, 2>(ctx, ham, a, grid);
-    case 3: return go_hub_size<T, C, 3>(ctx, ham, a, grid);
+    case 0: return go_hub_size<T, I, C, 0>(ctx, ham, a, grid);
+    case 1: return go_hub_size<T, I, C, 1>(ctx, ham, a, grid);
+    case 2: return go_hub_size<T, I, C, 2>(ctx, ham, a, grid);
+    case 3: return go_hub_size<T, I, C, 3>(ctx, ham, a, grid);
     default: return HPHI_E_INVAL;
     }
 }
@@ -408,7 +440,7 @@ int go_hub_red(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int red_m
 // Fixed-point diagonal tables of the Hubbard kernel.  ham->hub stays null when
 // the packed down-hop lists are missing, or the rows of one up string (16 bytes
 // per down string) do not fit in shared memory, or the model has more than 32
-// sites or 2^32 rows.
+// sites or 2^32 rows, or no integers hold its diagonal.
 int build_hub_tables(hphi_ctx *ctx, hphi_ham *H) {
     const hphi_basis *B = H->basis;
     if (B->model != HPHI_HUBBARD || B->N > 32 || H->D >= ((int64_t)1 << 32)) return HPHI_OK;
@@ -421,47 +453,89 @@ int build_hub_tables(hphi_ctx *ctx, hphi_ham *H) {
     g.up_pad = (H->up_w + 7) & ~7;  // whole batches of up hops
     g.ngrp = (B->N + kHubGroup - 1) / kHubGroup;
     g.nv = H->host.n_v;
-    if (std::max(hub_smem<double, 1>(g, H->host.n_ncoef), hub_smem<float, 1>(g, H->host.n_ncoef)) > 222 * 1024)
-        return HPHI_OK;
-    // |diagonal| <= sum |U| + 4 sum |V| < 2^e2; fixed point: 2^(59 - e2) per unit
-    double bound = 0.0;
-    for (int i = 0; i < B->N; i++) bound += fabs(H->host.U[i]);
-    for (int k = 0; k < g.nv; k++) bound += 4.0 * fabs(H->host.v[k].v);
-    if (!isfinite(bound)) return HPHI_OK;
-    int e2 = 0;
-    frexp(bound > 0.0 ? bound : 1.0, &e2);
-    g.scale64 = ldexp(1.0, e2 - 59);
-    g.scale32 = ldexp(1.0, e2 - 59 + kFixShift);
-    auto fixed = [&](double v) { return (long long)llrint(ldexp(v, 59 - e2)); };
-    std::vector<long long> blob(32, 0);  // ufix | vfix | per-species V parts
-    for (int i = 0; i < B->N; i++) blob[i] = fixed(H->host.U[i]);
-    std::vector<HubV> vf;
-    for (int k = 0; k < g.nv; k++) vf.push_back(HubV{H->host.v[k].i, H->host.v[k].j, fixed(H->host.v[k].v)});
-    const size_t at_v = blob.size();
-    blob.resize(at_v + vf.size() * (sizeof(HubV) / sizeof(long long)), 0);
-    if (!vf.empty()) memcpy(blob.data() + at_v, vf.data(), vf.size() * sizeof(HubV));
-    size_t at[2] = {0, 0};
-    if (g.nv > 0)  // V n_i n_j of one species alone, per string
+    // |U part| <= sum |U|, |V part| <= 4 sum |V|, each (or both together) below 2^e2;
+    // fixed point: 2^(62 - e2) per unit, the upper 32 bits of that in 32-bit integers
+    double ubound = 0.0, vbound = 0.0, hop = 0.0;
+    for (int i = 0; i < B->N; i++) ubound += fabs(H->host.U[i]);
+    for (int k = 0; k < g.nv; k++) vbound += 4.0 * fabs(H->host.v[k].v);
+    for (int k = 0; k < H->host.n_ncoef; k++) hop = k ? std::min(hop, fabs(H->host.coef[k])) : fabs(H->host.coef[k]);
+    if (!isfinite(ubound + vbound)) return HPHI_OK;
+    auto grid = [](double b) {
+        int e2 = 0;
+        frexp(b > 0.0 ? b : 1.0, &e2);
+        return e2;
+    };
+    const int eu = grid(ubound), ev = grid(vbound), e2 = grid(ubound + vbound);
+    if (std::min(eu, ev) < -60 || e2 > 100) return HPHI_OK;  // the scales are normal numbers in FP32 too
+    // Which integers: every coupling keeps the digits that it has in the vectors' type, or
+    // a grid step is at most a quarter ulp of the smallest hop, whose terms round by more
+    // (a row without U in its diagonal still gets hops).  V = 0.3 next to U = 100 on 14
+    // sites: off by 1.2e-6 of it on a 32-bit grid, 3e-16 on the same grid in 64 bits, 1e-18
+    // on its own.  ms per product of the 7x2 ladder with V, FP32: 32 bits 0.154, 64 bits
+    // 0.165, bond-major kernel 0.448; FP64: one grid 0.697, two 0.763, bond-major 1.075.
+    auto keeps = [&](int eu, int ev, int bits, int digits) {
+        bool ok = true;
+        for (int i = 0; i < B->N; i++) ok = ok && fix_keeps(H->host.U[i], eu, bits, digits);
+        for (int k = 0; k < g.nv; k++) ok = ok && fix_keeps(H->host.v[k].v, ev, bits, digits);
+        return ok || ldexp(1.0, std::max(eu, ev) - bits) <= ldexp(hop, -digits - 1);
+    };
+    const size_t most = 222 * 1024;
+    g.fix[0].parts = g.fix[1].parts = 1;
+    if (keeps(e2, e2, kHubBits, 53)) {
+        g.fix[1].bytes = 8;
+    } else if (g.nv > 0 && keeps(eu, ev, kHubBits, 53)) {
+        g.fix[1].bytes = 8;
+        g.fix[1].parts = 2;
+    }
+    if (g.fix[1].bytes && hub_smem<double, 1>(g, H->host.n_ncoef, 8) > most) g.fix[1].bytes = 0;
+    if (keeps(e2, e2, 30, 24)) g.fix[0].bytes = 4;
+    else if (keeps(e2, e2, kHubBits, 24)) g.fix[0].bytes = 8;
+    if (g.fix[0].bytes && hub_smem<float, 1>(g, H->host.n_ncoef, g.fix[0].bytes) > most) g.fix[0].bytes = 0;
+    if (!g.fix[0].bytes && !g.fix[1].bytes) return HPHI_OK;
+    std::vector<uint32_t> st[2];
+    if (g.nv > 0)
         for (int s = 0; s < 2; s++) {
-            const Species &sp = B->sp[s];
-            std::vector<uint32_t> st((size_t)sp.dim);
-            HPHI_CUDA(ctx, cudaMemcpy(st.data(), sp.states, st.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost));
-            at[s] = blob.size();
-            for (uint32_t x : st) {
+            st[s].resize((size_t)B->sp[s].dim);
+            HPHI_CUDA(ctx, cudaMemcpy(st[s].data(), B->sp[s].states, st[s].size() * sizeof(uint32_t),
+                                      cudaMemcpyDeviceToHost));
+        }
+    std::vector<long long> blob;  // per precision: ufix | vfix | V of one species alone, per string
+    size_t at_v[2], at_s[2][2];
+    for (int t = 0; t < 2; t++) {
+        const bool own = g.fix[t].parts == 2;
+        const int tu = own ? eu : e2, tv = own ? ev : e2;
+        auto fixed = [](double v, int e) { return (long long)llrint(ldexp(v, kHubBits - e)); };
+        const size_t at_u = blob.size();
+        blob.resize(at_u + 32, 0);
+        for (int i = 0; i < B->N; i++) blob[at_u + i] = fixed(H->host.U[i], tu);
+        std::vector<HubV> vf;
+        for (int k = 0; k < g.nv; k++) vf.push_back(HubV{H->host.v[k].i, H->host.v[k].j, fixed(H->host.v[k].v, tv)});
+        at_v[t] = blob.size();
+        blob.resize(at_v[t] + vf.size() * (sizeof(HubV) / sizeof(long long)), 0);
+        if (!vf.empty()) memcpy(blob.data() + at_v[t], vf.data(), vf.size() * sizeof(HubV));
+        for (int s = 0; s < 2; s++) {
+            at_s[t][s] = blob.size();
+            for (uint32_t x : st[s]) {
                 long long d = 0;
                 for (const HubV &v : vf)
                     if (((x >> v.i) & 1u) && ((x >> v.j) & 1u)) d += v.v;
                 blob.push_back(d);
             }
         }
+        const int bits = g.fix[t].bytes == 4 ? 30 : kHubBits;
+        g.fix[t].scale = ldexp(1.0, tu - bits);
+        g.fix[t].vscale = ldexp(1.0, tv - bits);
+    }
     cudaError_t e = cudaMalloc((void **)&H->hub_tab, blob.size() * sizeof(long long));
     if (e == cudaSuccess)
         e = cudaMemcpy(H->hub_tab, blob.data(), blob.size() * sizeof(long long), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_err(ctx, e, "Hubbard kernel tables");
-    g.ufix = H->hub_tab;
-    g.vfix = (const HubV *)(H->hub_tab + at_v);
-    g.dup = g.nv > 0 ? H->hub_tab + at[0] : nullptr;
-    g.ddnf = g.nv > 0 ? H->hub_tab + at[1] : nullptr;
+    for (int t = 0; t < 2; t++) {
+        g.fix[t].ufix = H->hub_tab + at_v[t] - 32;
+        g.fix[t].vfix = (const HubV *)(H->hub_tab + at_v[t]);
+        g.fix[t].dup = g.nv > 0 ? H->hub_tab + at_s[t][0] : nullptr;
+        g.fix[t].ddnf = g.nv > 0 ? H->hub_tab + at_s[t][1] : nullptr;
+    }
     H->hub = new (std::nothrow) HubArgs(g);
     if (!H->hub) return set_err(ctx, HPHI_E_NOMEM, "Hubbard kernel tables");
     return HPHI_OK;
@@ -470,8 +544,16 @@ int build_hub_tables(hphi_ctx *ctx, hphi_ham *H) {
 template <typename T>
 int launch_hub(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int red_mode, int *grid) {
     if (!ham->hub) return set_err(ctx, HPHI_E_INVAL, "Hubbard H*x: not available for this Hamiltonian");
-    if (a.ncol == 1) return go_hub_red<T, 1>(ctx, ham, a, red_mode, grid);
-    return go_hub_red<T, 2>(ctx, ham, a, red_mode, grid);
+    const int bytes = ham->hub->fix[sizeof(T) == 8].bytes;
+    if (bytes == 8) {
+        if (a.ncol == 1) return go_hub_red<T, long long, 1>(ctx, ham, a, red_mode, grid);
+        return go_hub_red<T, long long, 2>(ctx, ham, a, red_mode, grid);
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (bytes == 4 && a.ncol == 1) return go_hub_red<T, int, 1>(ctx, ham, a, red_mode, grid);
+        if (bytes == 4) return go_hub_red<T, int, 2>(ctx, ham, a, red_mode, grid);
+    }
+    return set_err(ctx, HPHI_E_INVAL, "Hubbard H*x: not available for this Hamiltonian");
 }
 
 template int launch_hub<float>(hphi_ctx *, const hphi_ham *, const HvArgs<float> &, int, int *);

@@ -60,6 +60,7 @@ constexpr int kLoadsU = 24, kLoadsM = 8;  // loads per lane in flight: uniform b
 // threads per block: one block per SM, registers for 32 (FP64: 16) warps
 template <typename T> constexpr int kSegThreads = sizeof(T) == 4 ? 1024 : 512;
 constexpr int kSegStage = 256;  // staged values per warp (a slot behind every segment stays 0)
+constexpr int kSegBits = 59;  // the diagonal lies below 2^59 grid steps
 constexpr int kSegRows = 8;   // rows of a lane held in registers (C(10, 5) = 252 rows per segment)
 
 // A bond of the image, in T's precision.
@@ -616,7 +617,7 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
     int e2 = 0;
     frexp(bound > 0.0 ? bound : 1.0, &e2);  // bound < 2^e2
     g.scale64 = ldexp(1.0, e2 - 61);
-    g.scale32 = ldexp(1.0, e2 - 61 + kFixShift);
+    g.scale32 = ldexp(1.0, e2 - 61 + kSegBits - 30);
     auto fixed = [&](double v) { return (long long)llrint(ldexp(v, 61 - e2)); };
     std::vector<WarpBond> ub, xb, ib;  // uniform, mixed, inner
     std::vector<std::vector<WarpBond>> mb(g.s);
@@ -740,12 +741,12 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
         const size_t at = blob.size();
         blob.resize(at + lay.bytes, 0);
         unsigned char *p = blob.data() + at;
-        for (int i = 0; i < rows; i++) ((typename FixInt<T>::type *)p)[i] = to_fix<T>(dl0[i]);
+        for (int i = 0; i < rows; i++) ((typename FixInt<T>::type *)p)[i] = to_fix<typename FixInt<T>::type, kSegBits>(dl0[i]);
         memcpy(p + lay.l0s, l0s.data(), sizeof(uint16_t) * rows);
         memcpy(p + lay.so, so.data(), sizeof(uint16_t) * so.size());
         memcpy(p + lay.jp, jp.data(), sizeof(uint32_t) * jp.size());
         for (size_t i = 0; i < all.size(); i++)
-            ((SmemBond<T> *)(p + lay.bonds))[i] = SmemBond<T>{(T)all[i].cxy, to_fix<T>(all[i].cz), all[i].mask, all[i].tab};
+            ((SmemBond<T> *)(p + lay.bonds))[i] = SmemBond<T>{(T)all[i].cxy, to_fix<typename FixInt<T>::type, kSegBits>(all[i].cz), all[i].mask, all[i].tab};
         if (!tall.empty()) memcpy(p + lay.tabs, tall.data(), tall.size());
         return at;
     };

@@ -92,3 +92,28 @@ def test_hubbard_kernel_pair_swap_and_reductions(dtype):
     want = m.lanczos(v0, 10, 0.0)
     assert np.allclose(got["alpha"], want["alpha"], atol=10 * tol) and np.allclose(got["beta"], want["beta"][1:],
                                                                                    atol=10 * tol)
+
+
+# One large coupling next to small ones: a row without a doubly occupied site (or without the
+# large U's) has only small terms in its diagonal, and x lives on such rows.
+@pytest.mark.parametrize("U", [1.0, 1e2, 1e4, 1e6, 1e8])
+@pytest.mark.parametrize("one_site", [False, True])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32, torch.complex128, torch.complex64])
+def test_small_couplings_next_to_a_large_one(U, one_site, dtype):
+    N = 8
+    terms = hubbard_terms(N, chain(N), t=1.0, U=0.3 if one_site else U, V=0.3)
+    if one_site:
+        terms.append(("HUBBARD_U", 2, 2, 0, U, 0.0))
+    m, b, h = pair("HUBBARD", N, 4, 3, terms)
+    up, dn = (s.cpu().numpy() for s in b.states(0, b.dim))
+    keep = ((up & dn) & ((1 << 2) if one_site else (1 << N) - 1)) == 0
+    cplx = dtype.is_complex
+    x = random_vectors(m.dim, 1, 11, complex_=cplx, normalize=False)[:, 0] * keep
+    xt = torch.from_numpy(x.copy()).to(dtype)
+    f = xt.to(torch.complex128 if cplx else torch.float64).numpy()
+    want = _h(m, f) if cplx else m.apply(f)
+    yd = torch.empty(m.dim, dtype=dtype, device="cuda")
+    hphi.hphi_apply_H(h, xt.cuda(), yd)
+    assert rel_err(yd.cpu().numpy(), want) < TOL[dtype]
+    if not cplx and dtype == torch.float32:
+        assert h.ctx.last_kernel().startswith("k_hub<f32,C1,64,I")
