@@ -8,10 +8,6 @@ namespace hphi {
 
 // A diagonal is an integer times a power of two, below 2^BITS in 64 bits; 32-bit
 // integers keep its upper bits (rounded), below 2^30.
-template <typename T>
-struct FixInt { using type = int; };
-template <>
-struct FixInt<double> { using type = long long; };
 
 // A 64-bit fixed-point value as an integer of type I.
 template <typename I, int BITS>

@@ -124,16 +124,20 @@ struct WarpClass {   // segments of one popcount: rows, rows per lane, offsets o
     uint32_t len;
     int nc, row0, tab;
 };
+struct WarpFix {                  // one precision of the vectors
+    int bytes;                    // integers that hold the diagonal: 8, 4 (the upper bits), 0 (no kernel)
+    double scale;                 // fixed point to value
+    const unsigned char *img;     // device: the tables' image (hv_warp.cu, WarpLayout)
+};
 struct WarpArgs {
     int s, n1, nlo, n, rot;
     int nu, nx, nm, ni;           // uniform, mixed, mixed diagonal, inner bonds
     int nrow, tab_stride, ntab;   // padded rows of all classes, bytes of a table, tables of the mixed bonds
-    double scale64, scale32;      // fixed point to value
+    WarpFix fix[2];               // FP32 vectors, FP64 vectors
     int moff[kWarpSegMax + 1];    // mixed diagonal entries of each segment bit
     uint8_t order[64];            // segments of a row block, long ones first
     WarpClass cls[kWarpSegMax + 1];
     int jl, jw, jhi;              // Lin's jb in two parts: low and high bits of h, 2^jw
-    const unsigned char *img32, *img64;  // device: the tables' images (hv_warp.cu, WarpLayout)
 };
 
 // Hubbard kernel (hv_hub.cu): sizes and the fixed-point diagonal.

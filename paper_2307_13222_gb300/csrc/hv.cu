@@ -318,7 +318,7 @@ int launch_typed(hphi_ctx *ctx, const hphi_ham *ham, HvLaunch &L) {
         // are longest (row blocks of 16 low bits: 4x8 56.9 against 62.3 ms; 15 bits: 6x5 15.5
         // against 15.2).  FP32 problems below 2^14 rows keep the bond-major kernel too: both
         // are one wave of latency there (16 sites: 10 us).
-        const bool warp = ham->tune_variant < 0 && ham->warp && one_col &&
+        const bool warp = ham->tune_variant < 0 && ham->warp && ham->warp->fix[sizeof(T) == 8].bytes && one_col &&
                           (std::is_same<T, double>::value ? ham->nlo < 16 : ham->D >= 16384);
         // Hubbard: one column or one aligned pair of columns (a complex vector), automatic where
         // its tables exist for the vectors' type (4x4 FP32 5.7 -> 3.4 ms, 6x2 complex FP64 0.149 -> 0.108 ms; 8 sites

@@ -21,11 +21,12 @@
 // accumulated through shared memory.
 //
 // The diagonal is summed in fixed point (integers, scaled by a power of two so
-// that it stays below 2^30, FP64 data 2^59; partial sums may wrap): the part of
+// that it stays below 2^30, in 64 bits 2^62; partial sums may wrap): the part of
 // u by one warp reduction, the mixed part from two 32-entry tables kept one
-// entry per lane (l0's low and high five bits), the part of l0 from a table.  A
-// coupling is rounded to 2^-32 (FP64 2^-61) of the sum of all |Jz|, less than
-// the T sums of the other kernels round, and it costs no FP64 adds.
+// entry per lane (l0's low and high five bits), the part of l0 from a table.  That
+// costs no FP64 adds.  A grid step is 2^-32 (2^-64) of a power of two above the sum
+// of all |Jz|, more than a weak coupling can do without where strong ones cancel:
+// build_warp_tables chooses the integers, or leaves the kernel out.
 //
 // Thread blocks take row blocks h (the high half of the spin string) in the
 // traversal order of set_traversal, the warps of a block its segments, so that
@@ -60,7 +61,7 @@ constexpr int kLoadsU = 24, kLoadsM = 8;  // loads per lane in flight: uniform b
 // threads per block: one block per SM, registers for 32 (FP64: 16) warps
 template <typename T> constexpr int kSegThreads = sizeof(T) == 4 ? 1024 : 512;
 constexpr int kSegStage = 256;  // staged values per warp (a slot behind every segment stays 0)
-constexpr int kSegBits = 59;  // the diagonal lies below 2^59 grid steps
+constexpr int kSegBits = 62;  // the diagonal lies below 2^62 grid steps
 constexpr int kSegRows = 8;   // rows of a lane held in registers (C(10, 5) = 252 rows per segment)
 
 // A bond of the image, in T's precision.
@@ -70,10 +71,10 @@ struct WarpBond {     // a bond as the builder collects it
     uint32_t mask;    // its sites above the segment bits
     uint32_t tab;     // rank table (mixed: of needed value 0; the next one of 1)
 };
-template <typename T>
+template <typename T, typename I>
 struct SmemBond {
     T cxy;
-    typename FixInt<T>::type cz;
+    I cz;
     uint32_t mask, tab;
 };
 
@@ -143,11 +144,11 @@ __device__ __forceinline__ void fma_rows(double c, const double (&v)[NC], double
 // diagonal, the segment strings, Lin offsets of the segments, jb in two parts,
 // the bonds (uniform, mixed, mixed diagonal, inner), the rank tables (mixed,
 // inner).  Every part is a multiple of 16 bytes.
-template <typename T>
+template <typename T, typename I>
 struct WarpLayout {
     uint32_t l0s, so, jp, bonds, tabs, bytes;
     __host__ __device__ explicit WarpLayout(const WarpArgs &g) {
-        uint32_t o = (uint32_t)sizeof(typename FixInt<T>::type) * g.nrow;
+        uint32_t o = (uint32_t)sizeof(I) * g.nrow;
         auto part = [&](uint32_t n) {
             const uint32_t at = o;
             o += (n + 15u) & ~15u;
@@ -156,19 +157,18 @@ struct WarpLayout {
         l0s = part(2u * g.nrow);
         so = part(2u * (uint32_t)((g.nlo + 1) << g.n1));
         jp = part(4u * (uint32_t)(g.jhi + ((g.jw + 1) << g.jl)));
-        bonds = part((uint32_t)sizeof(SmemBond<T>) * (g.nu + g.nx + g.nm + g.ni));
+        bonds = part((uint32_t)sizeof(SmemBond<T, I>) * (g.nu + g.nx + g.nm + g.ni));
         tabs = part((uint32_t)g.tab_stride * (g.ntab + g.ni));
         bytes = o;
     }
 };
 
 // What a warp needs to know of its segment.
-template <typename T>
+template <typename T, typename I>
 struct Seg {
-    using I = typename FixInt<T>::type;
     const SegEnt<T> *list;        // mixed bonds, then the applicable uniform ones
     int nml, nall;
-    const SmemBond<T> *ib;        // inner bonds
+    const SmemBond<T, I> *ib;        // inner bonds
     int nib;
     const unsigned char *tabs;    // rank tables of the mixed bonds, this class
     const unsigned char *itabs;   // rank tables of the inner bonds, this class
@@ -234,10 +234,9 @@ __device__ __forceinline__ void seg_out(const HvArgs<T> &a, const Epi<T> &e, uin
 // The rows of one segment, NC = ceil(len / 32) per lane.  Loads of whole rows of
 // 32 run past the segment's end into the rows behind it (whose sums are not
 // stored): the caller has checked that they stay inside x.
-template <typename T, int NC, int RED>
-__device__ __forceinline__ void seg_rows(const HvArgs<T> &a, const Seg<T> &g, const Epi<T> &e, int lane,
+template <typename T, typename I, int NC, int RED>
+__device__ __forceinline__ void seg_rows(const HvArgs<T> &a, const Seg<T, I> &g, const Epi<T> &e, int lane,
                                          RedAcc<T> (&racc)[RED == 2 ? 3 : 1]) {
-    using I = typename FixInt<T>::type;
     constexpr int UB = kLoadsU / NC, UM = kLoadsM / NC;  // uniform and mixed bonds in flight
     const T *__restrict__ xs = a.x + g.base;
     const T *__restrict__ xl = xs + lane;
@@ -325,10 +324,9 @@ __device__ __forceinline__ void seg_rows(const HvArgs<T> &a, const Seg<T> &g, co
 
 // The same for segments whose padded rows would reach past the end of x: 32
 // rows at a time, every access predicated, inner bonds read from x.
-template <typename T, int RED>
-__device__ __noinline__ void seg_edge(const HvArgs<T> &a, const Seg<T> &g, const Epi<T> &e, int lane, int nc,
+template <typename T, typename I, int RED>
+__device__ __noinline__ void seg_edge(const HvArgs<T> &a, const Seg<T, I> &g, const Epi<T> &e, int lane, int nc,
                                       RedAcc<T> (&racc)[RED == 2 ? 3 : 1]) {
-    using I = typename FixInt<T>::type;
     const T *__restrict__ xs = a.x + g.base;
     const int nb = nc > 4 ? 8 : nc > 2 ? 4 : nc;  // entries of a lane in the tables
     for (int c = 0; c < nc; c++) {
@@ -352,28 +350,27 @@ __device__ __noinline__ void seg_edge(const HvArgs<T> &a, const Seg<T> &g, const
     }
 }
 
-template <typename T, int RED, int NT, int MINB>
+template <typename T, typename I, int RED, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
     k_hvw(const __grid_constant__ HvArgs<T> a, const __grid_constant__ WarpArgs g) {
-    using I = typename FixInt<T>::type;
     constexpr int W = NT / 32;
     extern __shared__ __align__(16) unsigned char s_raw[];
     // shared layout: per warp the bond list and the staged segment, then the
     // Hamiltonian's tables (one copy of the image in memory), then the traversal
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nlist = g.nu + g.nx;
-    const WarpLayout<T> lay(g);
+    const WarpLayout<T, I> lay(g);
     SegEnt<T> *lists = (SegEnt<T> *)s_raw;
     T *stages = (T *)(s_raw + sizeof(SegEnt<T>) * (size_t)W * nlist);
     unsigned char *img = (unsigned char *)(stages + W * kSegStage);
     const I *dl0 = (const I *)img;
     const uint16_t *l0s = (const uint16_t *)(img + lay.l0s), *so = (const uint16_t *)(img + lay.so);
     const uint32_t *jp = (const uint32_t *)(img + lay.jp);
-    const SmemBond<T> *ub = (const SmemBond<T> *)(img + lay.bonds), *mb = ub + nlist, *ib = mb + g.nm;
+    const SmemBond<T, I> *ub = (const SmemBond<T, I> *)(img + lay.bonds), *mb = ub + nlist, *ib = mb + g.nm;
     const unsigned char *tabs = img + lay.tabs;
     uint16_t *perm = (uint16_t *)(img + lay.bytes);  // counter bytes to bits of h
     {
-        const uint4 *src = (const uint4 *)(sizeof(T) == 4 ? g.img32 : g.img64);
+        const uint4 *src = (const uint4 *)g.fix[sizeof(T) == 8].img;
 #pragma unroll 4
         for (int i = threadIdx.x; i < (int)(lay.bytes / 16); i += NT) ((uint4 *)img)[i] = __ldg(src + i);
         if (a.P.use_perm)
@@ -383,7 +380,7 @@ __global__ void __launch_bounds__(NT, MINB)
     __syncthreads();
     const T al = (T)(a.alpha_dev ? a.alpha_dev[0] : a.alpha[0]);
     if constexpr (RED != 2) {  // alpha goes into the coefficients (RED 2 needs H x itself)
-        for (int i = threadIdx.x; i < nlist + g.nm + g.ni; i += NT) ((SmemBond<T> *)ub)[i].cxy *= al;
+        for (int i = threadIdx.x; i < nlist + g.nm + g.ni; i += NT) ((SmemBond<T, I> *)ub)[i].cxy *= al;
         __syncthreads();
     }
     Epi<T> e;
@@ -392,10 +389,10 @@ __global__ void __launch_bounds__(NT, MINB)
     e.al = al;
     e.ga = (T)(a.gamma_dev ? a.gamma_dev[0] : a.gamma[0]);
     e.be = (T)a.beta;
-    e.dscale = (T)(sizeof(T) == 4 ? g.scale32 : g.scale64) * (RED != 2 ? al : (T)1);
+    e.dscale = (T)g.fix[sizeof(T) == 8].scale * (RED != 2 ? al : (T)1);
     e.use_beta = a.beta != 0.0;
     e.use_v = a.v != nullptr;
-    Seg<T> sg;
+    Seg<T, I> sg;
     SegEnt<T> *list = lists + (size_t)warp * nlist;
     sg.list = list;
     sg.nml = g.nx;
@@ -449,7 +446,7 @@ __global__ void __launch_bounds__(NT, MINB)
             bool app = false;
             SegEnt<T> n;
             if (k < nlist) {
-                const SmemBond<T> b = ub[k];
+                const SmemBond<T, I> b = ub[k];
                 const uint32_t m = S & b.mask;
                 const bool uni = k < g.nu, differ = m != 0 && m != b.mask;
                 if (!uni || differ) {
@@ -501,21 +498,21 @@ __global__ void __launch_bounds__(NT, MINB)
         sg.l0s = l0s + cl.row0;
         sg.itabs = tabs + (size_t)g.tab_stride * g.ntab + cl.tab;
         if (edge) {
-            const Seg<T> sg2 = sg;  // copies: what is passed by address lives in memory
+            const Seg<T, I> sg2 = sg;  // copies: what is passed by address lives in memory
             const Epi<T> e2 = e;
             RedAcc<T> r2[RED == 2 ? 3 : 1];
             for (int r = 0; r < NR; r++) r2[r] = racc[r];
-            seg_edge<T, RED>(a, sg2, e2, lane, cl.nc, r2);
+            seg_edge<T, I, RED>(a, sg2, e2, lane, cl.nc, r2);
             for (int r = 0; r < NR; r++) racc[r] = r2[r];
             continue;
         }
         switch (cl.nc) {
-        case 1: seg_rows<T, 1, RED>(a, sg, e, lane, racc); break;
-        case 2: seg_rows<T, 2, RED>(a, sg, e, lane, racc); break;
-        case 3: seg_rows<T, 3, RED>(a, sg, e, lane, racc); break;
-        case 4: seg_rows<T, 4, RED>(a, sg, e, lane, racc); break;
-        case 7: seg_rows<T, 7, RED>(a, sg, e, lane, racc); break;
-        default: seg_rows<T, 8, RED>(a, sg, e, lane, racc); break;
+        case 1: seg_rows<T, I, 1, RED>(a, sg, e, lane, racc); break;
+        case 2: seg_rows<T, I, 2, RED>(a, sg, e, lane, racc); break;
+        case 3: seg_rows<T, I, 3, RED>(a, sg, e, lane, racc); break;
+        case 4: seg_rows<T, I, 4, RED>(a, sg, e, lane, racc); break;
+        case 7: seg_rows<T, I, 7, RED>(a, sg, e, lane, racc); break;
+        default: seg_rows<T, I, 8, RED>(a, sg, e, lane, racc); break;
         }
     }
     if constexpr (RED != 0) {
@@ -539,42 +536,55 @@ __global__ void __launch_bounds__(NT, MINB)
     }
 }
 
-template <typename T>
+template <typename T, typename I>
 size_t warp_smem(const WarpArgs &g, int W) {
-    const WarpLayout<T> lay(g);
+    const WarpLayout<T, I> lay(g);
     return (sizeof(SegEnt<T>) * (size_t)(g.nu + g.nx) + sizeof(T) * kSegStage) * W + lay.bytes + 512 * sizeof(uint16_t);
 }
 
-template <typename T, int RED, int NT, int MINB>
+template <typename T, typename I, int RED, int NT, int MINB>
 int go_w(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int64_t want, int *grid_out) {
     const WarpArgs &g = *ham->warp;
-    const size_t dyn = warp_smem<T>(g, NT / 32);
-    const int occ = dyn_occupancy(ctx, (const void *)k_hvw<T, RED, NT, MINB>, NT, dyn);
+    const size_t dyn = warp_smem<T, I>(g, NT / 32);
+    const int occ = dyn_occupancy(ctx, (const void *)k_hvw<T, I, RED, NT, MINB>, NT, dyn);
     if (occ < 1) return set_err(ctx, HPHI_E_INVAL, "segment H*x: the tables do not fit in shared memory");
     // no more thread blocks than the partials of an H*x launch hold (8 per SM, one per row block)
     int64_t gr = std::min<int64_t>({(int64_t)std::min(occ, 8) * ctx->sm_count, ham->nh, want});
     if (gr < 1) gr = 1;
     *grid_out = (int)gr;
     const int slot = prof_begin(ctx, PROF_HV);
-    k_hvw<T, RED, NT, MINB><<<(int)gr, NT, dyn, ctx->stream>>>(a, g);
-    snprintf(ctx->last_kernel, sizeof ctx->last_kernel, "k_hvw<%s,%d,s%d,RED%d>@" HPHI_SRC_TAG, tname<T>(), NT, g.s, RED);
+    k_hvw<T, I, RED, NT, MINB><<<(int)gr, NT, dyn, ctx->stream>>>(a, g);
+    snprintf(ctx->last_kernel, sizeof ctx->last_kernel, "k_hvw<%s,%d,s%d,I%d,RED%d>@" HPHI_SRC_TAG, tname<T>(), NT, g.s,
+             (int)sizeof(I) * 8, RED);
     prof_end(ctx, slot);
     HPHI_CUDA(ctx, cudaGetLastError());
     return HPHI_OK;
 }
 
-template <typename T, int RED>
+template <typename T, typename I, int RED>
 int go_size(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int *grid) {
     const int64_t units = ham->nh << ham->warp->n1;
-    if (units >= (int64_t)ctx->sm_count * 64) return go_w<T, RED, kSegThreads<T>, 1>(ctx, ham, a, units, grid);
-    return go_w<T, RED, 64, 8>(ctx, ham, a, (units + 1) / 2, grid);
+    if (units >= (int64_t)ctx->sm_count * 64) return go_w<T, I, RED, kSegThreads<T>, 1>(ctx, ham, a, units, grid);
+    return go_w<T, I, RED, 64, 8>(ctx, ham, a, (units + 1) / 2, grid);
+}
+
+template <typename T, typename I>
+int go_red(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int red_mode, int *grid) {
+    switch (red_mode) {
+    case 0: return go_size<T, I, 0>(ctx, ham, a, grid);
+    case 1: return go_size<T, I, 1>(ctx, ham, a, grid);
+    case 2: return go_size<T, I, 2>(ctx, ham, a, grid);
+    case 3: return go_size<T, I, 3>(ctx, ham, a, grid);
+    default: return HPHI_E_INVAL;
+    }
 }
 
 }  // namespace
 
 // Tables of the segment kernel for a spin S^z-sector Hamiltonian of at most 32
 // sites and fewer than 2^31 rows (ham->warp stays null otherwise, or when the
-// tables would not fit in shared memory next to the bond lists).
+// tables would not fit in shared memory next to the bond lists, or when no integers
+// hold the diagonal).
 int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
     const hphi_basis *B = H->basis;
     if (B->model != HPHI_SPIN_HALF || B->N > 32 || H->nlo > 16 || H->nlo < 1 || H->D >= ((int64_t)1 << 31))
@@ -610,15 +620,32 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
         rows += 32 * (need > 4 ? 8 : need > 2 ? 4 : need);
     }
     g.nrow = g.tab_stride = rows;
-    // bonds; the diagonal (at most a quarter of sum |Jz|) in fixed point below 2^59
-    double bound = 0.0;
-    for (const DTerm &t : H->dterms) bound += fabs(t.a);
+    // bonds; the diagonal (at most a quarter of sum |Jz|) in fixed point below 2^62
+    double bound = 0.0, c0 = 0.0, weak = 0.0;  // weak: the smallest Jxy/2
+    for (const DTerm &t : H->dterms) {
+        bound += fabs(t.a);
+        c0 += 0.25 * t.a;
+        if (t.b != 0.0 && (weak == 0.0 || 0.5 * fabs(t.b) < weak)) weak = 0.5 * fabs(t.b);
+    }
     if (!isfinite(bound)) return HPHI_OK;
-    int e2 = 0;
-    frexp(bound > 0.0 ? bound : 1.0, &e2);  // bound < 2^e2
-    g.scale64 = ldexp(1.0, e2 - 61);
-    g.scale32 = ldexp(1.0, e2 - 61 + kSegBits - 30);
-    auto fixed = [&](double v) { return (long long)llrint(ldexp(v, 61 - e2)); };
+    int ed = 0;
+    frexp(bound > 0.0 ? 0.25 * bound : 1.0, &ed);  // |diagonal| < 2^ed
+    if (ed < -60 || ed > 100) return HPHI_OK;      // the scale is a normal number in FP32 too
+    // Which integers hold it: the grid follows the sum of all |Jz|, and strong bonds may
+    // cancel in a row.  Every Jz/2 keeps the digits that it has in the vectors' type, or a
+    // grid step is at most a quarter ulp of the smallest exchange coefficient, whose terms
+    // round by more; FP64 also where C0 = sum Jz/4 is not small against the grid (2^56
+    // steps), as the other kernels' sums start from C0 and round at its scale.  32-bit
+    // integers for FP32 vectors, 64-bit where those do not keep the digits (ms, 32, 64 bits,
+    // bond-major kernel: 14-rung ladder 0.493, 0.557, 1.58; 4x8 14.2, 14.6, 24.4).
+    auto keeps = [&](int bits, int digits) {
+        bool ok = true;
+        for (const DTerm &t : H->dterms) ok = ok && fix_keeps(0.5 * t.a, ed, bits, digits);
+        return ok || ldexp(1.0, ed - bits) <= ldexp(weak, -digits - 1);
+    };
+    if (keeps(kSegBits, 53) || fabs(c0) >= ldexp(1.0, ed - 6)) g.fix[1].bytes = 8;
+    g.fix[0].bytes = keeps(30, 24) ? 4 : keeps(kSegBits, 24) ? 8 : 0;
+    auto fixed = [&](double v) { return (long long)llrint(ldexp(v, kSegBits - ed)); };
     std::vector<WarpBond> ub, xb, ib;  // uniform, mixed, inner
     std::vector<std::vector<WarpBond>> mb(g.s);
     std::vector<int> tab_bit(g.s, -1);
@@ -636,7 +663,6 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
         to.push_back(t);
         return (uint32_t)to.size() - 1;
     };
-    double c0 = 0.0;
     std::vector<long long> dl0(rows, 0);
     std::vector<uint16_t> l0s(rows, 0);
     for (int c = 0; c <= g.s; c++)
@@ -644,7 +670,6 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
     for (const DTerm &t : H->dterms) {
         const int i = t.i < t.j ? t.i : t.j, j = t.i < t.j ? t.j : t.i;
         const double cz = -0.5 * t.a, cxy = 0.5 * t.b;
-        c0 += 0.25 * t.a;
         WarpBond b{};
         b.cxy = cxy;
         b.cz = fixed(cz);
@@ -730,32 +755,41 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
         return std::abs(2 * __builtin_popcount(x) - g.n1) < std::abs(2 * __builtin_popcount(y) - g.n1);
     });
     for (int i = 0; i < (1 << g.n1); i++) g.order[i] = (uint8_t)ord[i];
-    if (warp_smem<double>(g, kSegThreads<double> / 32) > 200 * 1024 ||
-        warp_smem<float>(g, kSegThreads<float> / 32) > 200 * 1024)
-        return HPHI_OK;
+    const size_t most = 200 * 1024;
+    if (warp_smem<double, long long>(g, kSegThreads<double> / 32) > most) g.fix[1].bytes = 0;
+    if ((g.fix[0].bytes == 8 ? warp_smem<float, long long>(g, kSegThreads<float> / 32)
+                             : warp_smem<float, int>(g, kSegThreads<float> / 32)) > most)
+        g.fix[0].bytes = 0;
+    if (!g.fix[0].bytes && !g.fix[1].bytes) return HPHI_OK;
     // the images of both precisions in one device block
     std::vector<unsigned char> blob;
-    auto image = [&](auto zero) {
+    auto image = [&](auto zero, auto izero) {
         using T = decltype(zero);
-        const WarpLayout<T> lay(g);
+        using I = decltype(izero);
+        const WarpLayout<T, I> lay(g);
         const size_t at = blob.size();
         blob.resize(at + lay.bytes, 0);
         unsigned char *p = blob.data() + at;
-        for (int i = 0; i < rows; i++) ((typename FixInt<T>::type *)p)[i] = to_fix<typename FixInt<T>::type, kSegBits>(dl0[i]);
+        for (int i = 0; i < rows; i++) ((I *)p)[i] = to_fix<I, kSegBits>(dl0[i]);
         memcpy(p + lay.l0s, l0s.data(), sizeof(uint16_t) * rows);
         memcpy(p + lay.so, so.data(), sizeof(uint16_t) * so.size());
         memcpy(p + lay.jp, jp.data(), sizeof(uint32_t) * jp.size());
         for (size_t i = 0; i < all.size(); i++)
-            ((SmemBond<T> *)(p + lay.bonds))[i] = SmemBond<T>{(T)all[i].cxy, to_fix<typename FixInt<T>::type, kSegBits>(all[i].cz), all[i].mask, all[i].tab};
+            ((SmemBond<T, I> *)(p + lay.bonds))[i] =
+                SmemBond<T, I>{(T)all[i].cxy, to_fix<I, kSegBits>(all[i].cz), all[i].mask, all[i].tab};
         if (!tall.empty()) memcpy(p + lay.tabs, tall.data(), tall.size());
         return at;
     };
-    const size_t at32 = image(0.0f), at64 = image(0.0);
+    size_t at[2] = {0, 0};
+    if (g.fix[0].bytes) at[0] = g.fix[0].bytes == 8 ? image(0.0f, 0ll) : image(0.0f, 0);
+    if (g.fix[1].bytes) at[1] = image(0.0, 0ll);
     cudaError_t e = cudaMalloc((void **)&H->warp_tab, blob.size());
     if (e == cudaSuccess) e = cudaMemcpy(H->warp_tab, blob.data(), blob.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_err(ctx, e, "segment kernel tables");
-    g.img32 = H->warp_tab + at32;
-    g.img64 = H->warp_tab + at64;
+    for (int t = 0; t < 2; t++) {
+        g.fix[t].img = H->warp_tab + at[t];
+        g.fix[t].scale = ldexp(1.0, ed - (g.fix[t].bytes == 4 ? 30 : kSegBits));
+    }
     H->warp = new (std::nothrow) WarpArgs(g);
     if (!H->warp) return set_err(ctx, HPHI_E_NOMEM, "segment kernel tables");
     return HPHI_OK;
@@ -766,13 +800,11 @@ int launch_warp(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int red_
     if (!ham->warp) return set_err(ctx, HPHI_E_INVAL, "segment H*x: not available for this Hamiltonian");
     if (a.ldx != 1 || a.ldy != 1 || (a.v && a.ldv != 1))
         return set_err(ctx, HPHI_E_INVAL, "segment H*x: one contiguous column only");
-    switch (red_mode) {
-    case 0: return go_size<T, 0>(ctx, ham, a, grid);
-    case 1: return go_size<T, 1>(ctx, ham, a, grid);
-    case 2: return go_size<T, 2>(ctx, ham, a, grid);
-    case 3: return go_size<T, 3>(ctx, ham, a, grid);
-    default: return HPHI_E_INVAL;
-    }
+    const int bytes = ham->warp->fix[sizeof(T) == 8].bytes;
+    if (bytes == 8) return go_red<T, long long>(ctx, ham, a, red_mode, grid);
+    if constexpr (sizeof(T) == 4)
+        if (bytes == 4) return go_red<T, int>(ctx, ham, a, red_mode, grid);
+    return set_err(ctx, HPHI_E_INVAL, "segment H*x: not available for this Hamiltonian");
 }
 
 template int launch_warp<float>(hphi_ctx *, const hphi_ham *, const HvArgs<float> &, int, int *);

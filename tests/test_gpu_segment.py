@@ -80,3 +80,25 @@ def test_segment_kernel_repeats_bitwise():
     a = hphi.hphi_lanczos(h, x, 30, 0.0, 30)
     c = hphi.hphi_lanczos(h, x, 30, 0.0, 30)
     assert (a["alpha"] == c["alpha"]).all() and (a["beta"] == c["beta"]).all()
+
+
+# Two strong Ising bonds that cancel on the rows where x lives, next to weak couplings: the
+# grid of the fixed-point diagonal follows the strong ones.  FP64: S first in the site order
+# and -S next, so that a sum over the bonds holds no trace of them.
+@pytest.mark.parametrize("S", [1.0, 1e4, 1e8])
+@pytest.mark.parametrize("dtype,pairs,sign,rows", [(torch.float32, ((0, 2), (4, 6)), -1, (0, 0)),
+                                                   (torch.float32, ((0, 2), (4, 6)), 1, (0, 1)),
+                                                   (torch.float64, ((0, 2), (0, 3)), -1, (0, 0))])
+def test_weak_couplings_next_to_cancelling_strong_ones(S, dtype, pairs, sign, rows):
+    N = 18
+    terms = [("XXZ", *pairs[0], 0, S, 0.0), ("XXZ", *pairs[1], 0, sign * S, 0.0)] + heisenberg_terms(chain(N)[1:], 0.7)
+    m, b, h = pair("SPIN_HALF", N, 9, 0, terms)
+    s = b.states(0, b.dim)[0].cpu().numpy()
+    anti = [((s >> i) ^ (s >> j)) & 1 for i, j in pairs]
+    x = random_vectors(m.dim, 1, 5, normalize=False)[:, 0] * ((anti[0] == rows[0]) & (anti[1] == rows[1]))
+    xt = torch.from_numpy(x).to(dtype)
+    y = torch.empty(m.dim, dtype=dtype, device="cuda")
+    hphi.hphi_apply_H(h, xt.cuda(), y)
+    assert rel_err(y.cpu().double().numpy(), m.apply(xt.double().numpy())) < TOL[dtype]
+    if dtype == torch.float32:
+        assert h.ctx.last_kernel().startswith("k_hvw<f32")
