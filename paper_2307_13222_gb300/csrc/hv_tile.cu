@@ -50,6 +50,7 @@
 #include "fixed.cuh"
 #include "hvcommon.cuh"
 
+#include <math.h>
 #include <string.h>
 
 #include <algorithm>
@@ -622,6 +623,7 @@ int build_tile_tables(hphi_ctx *ctx, hphi_ham *H, int prec) {
     std::vector<TileBond> bonds;
     for (const DTerm &t : H->dterms) {
         if (t.kind != DT_SPIN || t.b == 0.0) continue;
+        if (!(fabs(t.b) < 1e30)) return HPHI_OK;  // FP32 rows that a bond does not touch add Jxy/2 times 0
         adj[t.i] |= 1ull << t.j;
         adj[t.j] |= 1ull << t.i;
         bonds.push_back(TileBond{t.i, t.j, 0.5 * t.b});

@@ -625,6 +625,7 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
     for (const DTerm &t : H->dterms) {
         bound += fabs(t.a);
         c0 += 0.25 * t.a;
+        if (!(fabs(t.b) < 1e30)) return HPHI_OK;  // rows that a bond does not touch add 0 times alpha Jxy/2
         if (t.b != 0.0 && (weak == 0.0 || 0.5 * fabs(t.b) < weak)) weak = 0.5 * fabs(t.b);
     }
     if (!isfinite(bound)) return HPHI_OK;

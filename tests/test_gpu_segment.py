@@ -102,3 +102,17 @@ def test_weak_couplings_next_to_cancelling_strong_ones(S, dtype, pairs, sign, ro
     assert rel_err(y.cpu().double().numpy(), m.apply(xt.double().numpy())) < TOL[dtype]
     if dtype == torch.float32:
         assert h.ctx.last_kernel().startswith("k_hvw<f32")
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("model,ncol", [("SPIN_HALF", 1), ("SPIN_HALF_GC", 32)])
+def test_coupling_that_is_not_finite_stays_on_its_rows(model, ncol, dtype):
+    """An infinite exchange coupling marks the rows of its bond and no others (segment and
+    tiled kernels)."""
+    N = 18 if ncol == 1 else 9
+    m, b, h = pair(model, N, N // 2, 0, heisenberg_terms(chain(N), 0.7)[1:] + [("XXZ", 0, 1, 0, 0.7, float("inf"))])
+    s = b.states(0, b.dim)[0].cpu().numpy()
+    x = torch.ones((m.dim, ncol), dtype=dtype, device="cuda")
+    y = torch.empty_like(x)
+    hphi.hphi_apply_H(h, x, y)
+    assert (np.isfinite(y.cpu().numpy()) == (((s ^ (s >> 1)) & 1) == 0)[:, None]).all()
