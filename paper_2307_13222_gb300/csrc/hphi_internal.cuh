@@ -156,6 +156,7 @@ struct HubFix {
 struct HubArgs {
     int N, up_pad, ngrp, nv;      // up_pad: most up hops of a string, padded to 8
     uint32_t nh, ddn;             // up and down strings
+    uint32_t split;               // thread blocks that share a group of up strings (set per launch)
     HubFix fix[2];                // FP32 vectors, FP64 vectors
 };
 

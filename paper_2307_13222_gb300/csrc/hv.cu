@@ -481,9 +481,10 @@ __global__ void __launch_bounds__(kSumThreads)
 
 size_t hv_partials_size(hphi_ctx *ctx, const hphi_ham *ham, int ncol) {
     // at most 2048 / kThreads resident blocks per SM, so no launch is larger
+    // nor larger than the row blocks (the Hubbard kernel splits few row blocks over the SMs)
     int64_t g = (int64_t)ctx->sm_count * (2048 / kThreads);
-    if (g > ham->nh) g = ham->nh;
-    if (g < 1) g = 1;
+    const int64_t most = ham->nh > ctx->sm_count ? ham->nh : ctx->sm_count;
+    if (g > most) g = most;
     return (size_t)g * 3 * (size_t)ncol;
 }
 

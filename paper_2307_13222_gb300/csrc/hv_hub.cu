@@ -101,6 +101,9 @@ __device__ __forceinline__ void hub_store(T *y, uint32_t r, const T (&v)[C]) {
 template <typename T>
 __host__ __device__ __forceinline__ int hub_parts(const HubArgs &g) { return sizeof(T) == 8 ? g.fix[1].parts : 1; }
 
+// dn strings of a thread at a time (an FP64 pair fills the pipe with one)
+template <typename T, int C> constexpr int hub_dn = sizeof(T) == 8 && C == 2 ? 1 : 2;
+
 // acc[i] += c v[i] over one pack
 __device__ __forceinline__ void pack_fma(float c, const HubPack<float> &v, float (&acc)[4]) {
 #pragma unroll
@@ -115,8 +118,7 @@ template <typename T, typename I, int C, int RED, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
     k_hub(const __grid_constant__ HvArgs<T> a, const __grid_constant__ HubArgs g) {
     constexpr int P = 16 / (int)sizeof(T), U = P / C;
-    // dn strings of a thread at a time (an FP64 pair fills the pipe with one)
-    constexpr int QB = sizeof(T) == 8 && C == 2 ? 1 : 2;
+    constexpr int QB = hub_dn<T, C>;
     constexpr int HB = 8 / C / ((int)sizeof(T) / 4);        // up hops in flight
     constexpr int DB = 4;                                   // down hops in flight
     extern __shared__ __align__(16) unsigned char s_raw[];
@@ -147,9 +149,10 @@ __global__ void __launch_bounds__(NT, MINB)
     const T *__restrict__ X = a.x;
     constexpr int NR = RED == 2 ? 3 : (RED ? 1 : 0);
     RedAcc<T> racc[NR > 0 ? NR : 1][C];
-    const uint32_t nblk = (g.nh + U - 1) / U;
+    // unit blk: U up strings and every g.split-th round of their down strings
+    const uint32_t nblk = (g.nh + U - 1) / U * g.split;
     for (uint32_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-        const uint32_t u0 = blk * U;
+        const uint32_t u0 = blk / g.split * U, part = blk % g.split;
         __syncthreads();  // the previous block is done with the shared arrays
         // up hops, down-site weights w_j = U_j n_j + sum V n_other, rows of the block
         for (int i = threadIdx.x; i < U * g.up_pad; i += NT) {
@@ -208,7 +211,7 @@ __global__ void __launch_bounds__(NT, MINB)
             tab[i] = s;
         }
         __syncthreads();
-        for (uint32_t q0 = threadIdx.x; q0 < ddn; q0 += NT * QB) {
+        for (uint32_t q0 = threadIdx.x + part * (NT * QB); q0 < ddn; q0 += NT * QB * g.split) {
             T acc[QB][P];
             uint32_t q[QB];
             bool on[QB];
@@ -400,13 +403,18 @@ size_t hub_smem(const HubArgs &g, int ncoef, int int_bytes) {
 
 template <typename T, typename I, int C, int RED, int NT, int MINB>
 int go_hub(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int *grid) {
-    const HubArgs &g = *ham->hub;
+    HubArgs g = *ham->hub;
     const size_t dyn = hub_smem<T, C>(g, ham->host.n_ncoef, (int)sizeof(I));
     const int occ = dyn_occupancy(ctx, (const void *)k_hub<T, I, C, RED, NT, MINB>, NT, dyn);
     if (occ < 1) return set_err(ctx, HPHI_E_INVAL, "Hubbard H*x: the rows of an up string do not fit in shared memory");
     constexpr int U = 16 / (int)sizeof(T) / C;
+    // few up strings: several thread blocks share them, each with a part of the down strings
+    // (they all stage the rows), as long as every one gets an SM and a round of its own
+    // (us: 16 sites, 1 up 7 down, FP64 180 -> 39, bond-major kernel 109; FP32 67 -> 20, 66)
+    const int64_t blocks = (g.nh + U - 1) / U, rounds = (g.ddn + NT * hub_dn<T, C> - 1) / (NT * hub_dn<T, C>);
+    g.split = (uint32_t)std::max<int64_t>(1, std::min<int64_t>(rounds, ctx->sm_count / blocks));
     // no more thread blocks than the partials of an H*x launch hold (8 per SM)
-    const int64_t gr = std::min<int64_t>((int64_t)std::min(occ, 8) * ctx->sm_count, (g.nh + U - 1) / U);
+    const int64_t gr = std::min<int64_t>((int64_t)std::min(occ, 8) * ctx->sm_count, blocks * g.split);
     *grid = (int)(gr < 1 ? 1 : gr);
     const int slot = prof_begin(ctx, PROF_HV);
     k_hub<T, I, C, RED, NT, MINB><<<*grid, NT, dyn, ctx->stream>>>(a, g);
@@ -419,6 +427,17 @@ int go_hub(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int *grid) {
 
 template <typename T, typename I, int C, int RED>
 int go_hub_size(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int *grid) {
+    // Where the blocks leave SMs or the wave half empty, wider ones run fewer rounds one after
+    // the other: 1024 threads up to one block per SM, 256 up to four, as far as the down
+    // strings fill them (FP64 real: two per thread keep the pipe busy up to 1024).  us: 14
+    // sites, 2 up 7 down, FP32 45 -> 16, bond-major kernel 31; 10 sites, 2 up 5 down, complex
+    // FP64 20.5 -> 9.9, generic kernel 12.4.
+    constexpr int U = 16 / (int)sizeof(T) / C;
+    const int64_t blocks = (ham->hub->nh + U - 1) / U, ddn = ham->hub->ddn;
+    if (blocks <= ctx->sm_count && ddn > (sizeof(T) == 8 && C == 1 ? 1024 : 512))
+        return go_hub<T, I, C, RED, 1024, 1>(ctx, ham, a, grid);
+    if (blocks <= 4 * ctx->sm_count && ddn > 64 && ddn <= 512)
+        return go_hub<T, I, C, RED, 256, 4>(ctx, ham, a, grid);
     if (ham->hub->ddn > 4096) return go_hub<T, I, C, RED, 1024, 1>(ctx, ham, a, grid);
     if (ham->hub->ddn > 512) return go_hub<T, I, C, RED, 256, 4>(ctx, ham, a, grid);
     return go_hub<T, I, C, RED, 64, 8>(ctx, ham, a, grid);

@@ -117,3 +117,32 @@ def test_small_couplings_next_to_a_large_one(U, one_site, dtype):
     assert rel_err(yd.cpu().numpy(), want) < TOL[dtype]
     if not cplx and dtype == torch.float32:
         assert h.ctx.last_kernel().startswith("k_hub<f32,C1,64,I")
+
+
+# Few up strings: wider thread blocks, several of which share a group of up strings (1 to 6 here,
+# more of them than up strings), the last with an incomplete round; the partial sums of all.
+@pytest.mark.parametrize("N,nu,nd,threads", [(14, 0, 7, 1024), (14, 1, 7, 1024), (13, 1, 6, 1024), (16, 1, 7, 1024),
+                                             (10, 2, 5, 256), (9, 8, 4, 256)])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32, torch.complex128, torch.complex64])
+def test_few_up_strings(N, nu, nd, threads, dtype):
+    m, b, h = pair("HUBBARD", N, nu, nd, hubbard_terms(N, chain(N), t=1.0, U=4.0, V=0.5))
+    cplx = dtype.is_complex
+    tol = TOL[dtype]
+    v0 = random_vectors(m.dim, 1, N + nd, complex_=cplx)
+    Vg = torch.from_numpy(v0[:, 0].copy()).to(dtype).cuda()
+    if cplx:
+        Vo = Vg.cpu().to(torch.complex128).numpy()[:, None].copy()
+        n2, e, h2, n2n = hphi.hphi_time_step(h, Vg, 0.02, 3)
+        no, eo, noo = m.time_step(Vo, 0.02, 3)
+        assert rel_err(Vg.cpu().numpy(), Vo[:, 0]) < 4 * tol
+        assert np.allclose(n2, no, rtol=4 * tol) and np.allclose(n2n, noo, rtol=4 * tol)
+        assert np.allclose(e, eo, rtol=4 * tol, atol=40 * tol)
+    else:
+        x = Vg.double().cpu().numpy()
+        got, want = hphi.hphi_lanczos(h, Vg, 3, 0.0, 3), m.lanczos(x, 3, 0.0)
+        assert np.allclose(got["alpha"], want["alpha"], atol=40 * tol)
+        assert np.allclose(got["beta"], want["beta"][1:], atol=40 * tol)
+        y = torch.empty_like(Vg)
+        hphi.hphi_apply_H(h, Vg, y)
+        assert rel_err(y.double().cpu().numpy(), m.apply(x)) < tol
+    assert f",{threads},I" in h.ctx.last_kernel() and h.ctx.last_kernel().startswith("k_hub<")
