@@ -588,20 +588,27 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
         }
     };
     const int nthreads = nprob >= 64 ? std::max(1, std::min(16, (int)std::thread::hardware_concurrency())) : 1;
-    // Large batches run one chunk ahead of the checks: the tridiagonal problems of 200 small
-    // solves take the host longer than 8 steps take the GPU (a problem that turns out to be
-    // finished ignores its extra steps).  Small batches wait for the check instead.
-    const bool ahead = nthreads > 1;
-    auto launch = [&](int k0) -> int {
+    // Large batches run up to 16 steps ahead of the checks: the tridiagonal problems of 200
+    // small solves take the host longer than 8 steps take the GPU (a problem that turns out
+    // to be finished ignores its extra steps).  The rest of a longer chunk waits for the
+    // check, so that a batch that is done has run no more than 16 steps too many.  Small
+    // batches wait for the check altogether.  (ms, 200 16-site chains in chunks of 8 / 25 /
+    // 100 steps: no step ahead 27.8 / 24.7 / 29.9, a whole chunk 20.2 / 22.2 / 39.4, 8 steps
+    // 20.3 / 21.0 / 29.2, 16 steps 20.4 / 21.5 / 29.1; 200 of 12 to 16 sites in chunks of 16:
+    // whole 15.2, 8 steps 16.5, 16 steps 15.1.)
+    const int ahead = nthreads > 1 ? std::min(chunk, 16) : 0;
+    auto launch = [&](int k0, int n) -> int {
+        n = std::min(n, M - k0);
+        if (n <= 0) return HPHI_OK;
         for (int p = 0; p < nprob; p++) {
             hp[p].k0 = k0;
-            hp[p].nsteps = done[p] ? 0 : std::min(chunk, M - k0);
+            hp[p].nsteps = done[p] ? 0 : n;
         }
         HPHI_CUDA(ctx, send());
         return batch_launch_steps(ctx, dprob, nprob, dyn_bytes);
     };
     int k = 0, left = nprob;
-    int stl = launch(0);
+    int stl = launch(0, chunk);
     if (stl) return fail(stl);
     while (left > 0 && k < M) {
         const int c = std::min(chunk, M - k);
@@ -615,7 +622,7 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
         HPHI_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         const int k_prev = k;
         k += c;
-        if (ahead && k < M && (stl = launch(k))) return fail(stl);
+        if ((stl = launch(k, ahead))) return fail(stl);
         if (nthreads == 1) {
             std::vector<double> ap, bp;
             for (int p = 0; p < nprob; p++)
@@ -632,7 +639,7 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
         }
         left = 0;
         for (int p = 0; p < nprob; p++) left += !done[p];
-        if (!ahead && left > 0 && k < M && (stl = launch(k))) return fail(stl);
+        if (left > 0 && (stl = launch(k + ahead, chunk - ahead))) return fail(stl);
     }
     // energies (eigenvalues of T_m) and, where asked for, the Ritz vector of T_m
     // for the ground-state pass; spread over host threads for large batches

@@ -109,3 +109,38 @@ def test_edge_cases():
         hphi.hphi_lanczos_batch([h], [torch.zeros(3, dtype=torch.float64, device="cuda")], 5, 1e-12)
     with pytest.raises(hphi.HphiError):  # refused by the library: FP64 only, checked before any launch
         opts_bad = hphi.hphi_lanczos_batch([h], [vs[1]], 0, 1e-12)
+
+
+def test_large_mixed_batch_equals_small_ones():
+    """65 problems of mixed models and sizes in ascending order (run ahead of the checks, long
+    problems first), vectors for some, with a zero start, an eigenvector, a one-state sector and
+    one that does not converge: bit for bit what the same problems give in batches of 13."""
+    specs = [("SPIN_HALF", 6, 6, 0, heisenberg_terms(chain(6), 1.3)), ("SPIN_HALF", 8, 4, 0, heisenberg_terms(chain(8), 1.0))]
+    specs += [("SPIN_HALF", 10, 5, 0, heisenberg_terms(chain(10), uniform_couplings(10, 0.5, 1.5, s))) for s in range(20)]
+    specs += [("HUBBARD", 6, 3, 2, hubbard_terms(6, chain(6), t=1.0, U=2.0 + s)) for s in range(20)]
+    specs += [("SPIN_HALF_GC", 10, 0, 0, heisenberg_terms(chain(10), uniform_couplings(10, 0.5, 1.5, 50 + s)))
+              for s in range(10)]
+    specs += [("SPIN_HALF", 13, 6, 0, heisenberg_terms(chain(13), uniform_couplings(13, 0.5, 1.5, 90 + s)))
+              for s in range(13)]
+    ms, hs, vs = _build([("", *s, 40 + i) for i, s in enumerate(specs)])
+    vs[2].zero_()
+    vs[1].copy_(torch.from_numpy(np.linalg.eigh(O.dense_matrix(ms[1]))[1][:, 0].copy()))
+    H = [h for _, h in hs]
+    keys = ("e0", "steps", "status", "breakdown", "resid", "resid_est")
+
+    def solve(sel, check, steps):
+        g = [torch.full_like(vs[p], float("nan")) if p % 3 else None for p in sel]
+        return hphi.hphi_lanczos_batch([H[p] for p in sel], [vs[p] for p in sel], steps, 1e-12, check, g), g
+
+    assert len(specs) == 65
+    for check, steps in ((8, 400), (50, 400), (3, 35)):
+        big, gb = solve(range(65), check, steps)
+        for part in range(5):
+            sel = range(13 * part, 13 * part + 13)
+            small, gs = solve(sel, check, steps)
+            for p, r, g in zip(sel, small, gs):
+                for k in keys:
+                    assert np.array_equal(big[p][k], r[k], equal_nan=True), (check, p, k, big[p][k], r[k])
+                assert g is None or torch.equal(g.nan_to_num(7.0), gb[p].nan_to_num(7.0)), (check, p)
+        assert big[2]["status"] == -1 and big[0]["breakdown"] and big[1]["steps"] == 1
+        assert steps == 400 or any(r["status"] == -4 for r in big)
