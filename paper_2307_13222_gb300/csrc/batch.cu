@@ -673,13 +673,14 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
             });
         for (auto &th : pool) th.join();
     }
-    // the Ritz vectors in one copy (with the per-problem scalars, which are spent by now)
-    std::vector<double> yall;
+    // the Ritz vectors in one copy, as many rows as the longest of them
+    size_t ylen = 0;
+    for (int p = 0; p < nprob; p++) ylen = std::max(ylen, yv[p].size());
+    std::vector<double> yall(ylen * nprob, 0.0);
     for (int p = 0; p < nprob; p++) {
         if (yv[p].empty()) continue;
-        if (yall.empty()) yall.assign(n_pp, 0.0);
         const int m = (int)yv[p].size();
-        std::copy(yv[p].begin(), yv[p].end(), yall.begin() + (size_t)p * (M + 2) + 2);
+        std::copy(yv[p].begin(), yv[p].end(), yall.begin() + (size_t)p * ylen);
         hp[p].m = m;
         hp[p].theta = theta[p];
         hp[p].gs = (double *)gs_out[p];
@@ -687,7 +688,8 @@ extern "C" int hphi_lanczos_batch(hphi_ctx *ctx, int nprob, hphi_ham *const *ham
     }
     std::vector<double> gres(nprob, -1.0);
     if (any_gs) {
-        HPHI_CUDA(ctx, cudaMemcpyAsync(pp, yall.data(), sizeof(double) * n_pp, cudaMemcpyHostToDevice, ctx->stream));
+        HPHI_CUDA(ctx, cudaMemcpy2DAsync(pp + 2, sizeof(double) * (M + 2), yall.data(), sizeof(double) * ylen,
+                                         sizeof(double) * ylen, nprob, cudaMemcpyHostToDevice, ctx->stream));
         HPHI_CUDA(ctx, send());
         int stg = batch_launch_gs(ctx, dprob, nprob, dyn_bytes);
         if (stg) return fail(stg);
