@@ -143,8 +143,7 @@ void free_ham(hphi_ham *h) {
     cudaFree(h->ph_off);
     cudaFree(h->dterms_d);
     cudaFree(h->rowstate);
-    cudaFree(h->seg_so);
-    cudaFree(h->warp_tab);
+    cudaFree(h->sector_tab);
     cudaFree(h->hub_tab);
     delete h->warp;
     delete h->hub;
@@ -181,41 +180,39 @@ int build_bond_lists(hphi_ctx *ctx, hphi_ham *H, const std::vector<LLBond> &ll, 
         pos[l] = (uint32_t)c.size();
         c.push_back(l);
     }
-    std::vector<uint32_t> ent;
+    // at most 2^N_lo entries per bond and per (low bit, need); every candidate is written and
+    // kept or not, and at[q] counts the entries below row q, so that no branch depends on
+    // the data (us to build the Hamiltonian with push_back and a search per boundary, and
+    // so: 20-site chain 185, 163; 14-rung ladder 1760, 1050)
+    std::vector<uint32_t> ent(((size_t)(nll + 2 * nlb) << nlo) + 1);
     std::vector<int32_t> off;
-    auto close_group = [&](size_t start, uint32_t len) {
-        size_t i = start;
-        for (int r = 0; r <= kPhRanges; r++) {
-            const uint32_t qb = (uint32_t)(((uint64_t)len * r) / kPhRanges);
-            while (i < ent.size() && (ent[i] & 0xFFFFu) < qb) i++;
-            off.push_back((int32_t)i);
-        }
-    };
-    for (int p = 0; p <= nlo; p++) {
-        const std::vector<uint32_t> &c = cls[p];
-        for (int k = 0; k < nll; k++) {
-            const size_t start = ent.size();
-            const uint32_t m = (1u << ll[k].i) | (1u << ll[k].j);
-            if (ll[k].cxy != 0.0)
-                for (uint32_t q = 0; q < c.size(); q++) {
-                    const uint32_t lm = c[q] & m;
-                    if (lm != 0 && lm != m) ent.push_back(q | pos[c[q] ^ m] << 16);
-                }
-            close_group(start, (uint32_t)c.size());
-        }
-    }
-    H->ph_mx0 = (int64_t)off.size();
-    for (int p = 0; p <= nlo; p++) {
-        const std::vector<uint32_t> &c = cls[p];
-        for (int bi = 0; bi < nlb; bi++)
-            for (uint32_t need = 0; need < 2; need++) {
-                const size_t start = ent.size();
-                const int b = lowbits[bi];
-                for (uint32_t q = 0; q < c.size(); q++)
-                    if (((c[q] >> b) & 1u) == need) ent.push_back(q | pos[c[q] ^ (1u << b)] << 16);
-                close_group(start, (uint32_t)c.size());
+    off.reserve((size_t)(nlo + 1) * (nll + 2 * nlb) * (kPhRanges + 1));
+    std::vector<int32_t> at(((size_t)1 << nlo) + 1);
+    size_t ne = 0;
+    // one group: the rows of class c whose bit i differs from bit j (or, j < 0, equals need)
+    // and the positions of l ^ flip
+    auto group = [&](const std::vector<uint32_t> &c, int i, int j, uint32_t need, uint32_t flip, bool any) {
+        const uint32_t len = (uint32_t)c.size();
+        if (any)
+            for (uint32_t q = 0; q < len; q++) {
+                const uint32_t l = c[q];
+                at[q] = (int32_t)ne;
+                ent[ne] = q | pos[l ^ flip] << 16;
+                ne += j < 0 ? (((l >> i) ^ need) & 1u) ^ 1u : ((l >> i) ^ (l >> j)) & 1u;
             }
-    }
+        else
+            for (uint32_t q = 0; q < len; q++) at[q] = (int32_t)ne;
+        at[len] = (int32_t)ne;
+        for (int r = 0; r <= kPhRanges; r++) off.push_back(at[((uint64_t)len * r) / kPhRanges]);
+    };
+    for (int p = 0; p <= nlo; p++)
+        for (int k = 0; k < nll; k++)
+            group(cls[p], ll[k].i, ll[k].j, 0u, (1u << ll[k].i) | (1u << ll[k].j), ll[k].cxy != 0.0);
+    H->ph_mx0 = (int64_t)off.size();
+    for (int p = 0; p <= nlo; p++)
+        for (int b = 0; b < nlb; b++)
+            for (uint32_t need = 0; need < 2; need++) group(cls[p], lowbits[b], -1, need, 1u << lowbits[b], true);
+    ent.resize(ne);
     if (ent.size() >= ((size_t)1 << 31)) return HPHI_OK;  // lists unavailable: the kernel is not offered
     int st;
     if ((st = to_dev(ctx, &H->ph_ent, ent)) || (st = to_dev(ctx, &H->ph_off, off))) return st;
@@ -317,7 +314,14 @@ int build_spin(hphi_ctx *ctx, hphi_ham *H, const hphi_term *terms, int n_terms) 
     cudaFree(d_lb);
     if (e != cudaSuccess) return cuda_err(ctx, e, "k_spin_tables");
     if (sector && nlo <= 16 && ll.size() <= 128 && (st = build_bond_lists(ctx, H, ll, lowbits))) return st;
-    if (sector && ((st = build_seg_tables(ctx, H)) || (st = build_warp_tables(ctx, H)))) return st;
+    if (!sector) return HPHI_OK;
+    std::vector<unsigned char> blob;
+    size_t at[3] = {0, 0, 0};
+    if ((st = build_warp_tables(ctx, H, blob, at + 1)) || (st = build_seg_tables(ctx, H, blob, at)) ||
+        (st = to_dev(ctx, &H->sector_tab, blob)))
+        return st;
+    if (H->seg) H->seg->so = (const uint16_t *)(H->sector_tab + at[0]);
+    for (int t = 0; H->warp && t < 2; t++) H->warp->fix[t].img = H->sector_tab + at[1 + t];
     return HPHI_OK;
 }
 

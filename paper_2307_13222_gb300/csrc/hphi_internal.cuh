@@ -117,6 +117,16 @@ struct SegArgs {
     const uint16_t *so;  // [(N_lo + 1) << n1]
 };
 
+// C(n, k) for n <= 32, 0 outside 0 <= k <= n (host tables).
+struct Binomials {
+    int64_t c[33][33] = {};
+    constexpr Binomials() {
+        for (int n = 0; n <= 32; n++)
+            for (int k = 0; k <= n; k++) c[n][k] = k == 0 || k == n ? 1 : c[n - 1][k - 1] + c[n - 1][k];
+    }
+    int64_t operator()(int n, int k) const { return k < 0 || k > n ? 0 : c[n][k]; }
+};
+
 // Segment kernel (hv_warp.cu): the lowest s bits form the segments, the other
 // n1 bits of the low half and the high half pick one.
 constexpr int kWarpSegMax = 10;  // most segment bits
@@ -149,7 +159,7 @@ struct HubFix {
     int bytes;                    // integers that hold it: 8, 4 (the upper bits), 0 (no kernel)
     int parts;                    // 2: V has a grid of its own (FP64)
     double scale, vscale;         // fixed point to value; of that V
-    const long long *ufix;        // device [32]: U per site
+    long long ufix[32];           // U per site
     const HubV *vfix;             // device [nv]
     const long long *dup, *ddnf;  // device: V terms of one species alone, per up / down string (null: none)
 };
@@ -248,15 +258,13 @@ struct hphi_ham {
     int32_t *ph_off = nullptr;
     int64_t ph_mx0 = 0;          // first offset row of the mixed-bond groups
     int max_row_entries = 0;
-    // high-high pass (spin S^z sector, N_lo <= 16): host copy of its
-    // arguments (null when not available) and its device table
+    // high-high pass (spin S^z sector, N_lo <= 16) and segment kernel (spin S^z
+    // sector): host copies of their arguments (null when not available) and the
+    // device tables of both
     hphi::SegArgs *seg = nullptr;
-    uint16_t *seg_so = nullptr;
-    // segment kernel (spin S^z sector): host copy of its arguments (null when not
-    // available) and its device tables
     hphi::WarpArgs *warp = nullptr;
-    unsigned char *warp_tab = nullptr;
-    // Hubbard kernel: its arguments (null when not available) and device tables
+    unsigned char *sector_tab = nullptr;
+    // Hubbard kernel: its arguments (null when not available) and device tables (V terms)
     hphi::HubArgs *hub = nullptr;
     long long *hub_tab = nullptr;
     // tiled block kernel (full space, 32 columns), per precision [0: FP32, 1: FP64]
@@ -391,9 +399,11 @@ int lowest_ritz_warm(int m, const double *alpha, const double *beta2, double *wa
 int lowest_vector(int m, const double *alpha, const double *beta2, double *theta, std::vector<double> &y);
 
 // ---- high-high pass table (hv_seg.cu) ------------------------------------------------
-int build_seg_tables(hphi_ctx *ctx, hphi_ham *H);
-// ---- segment kernel tables (hv_warp.cu) ----------------------------------------------
-int build_warp_tables(hphi_ctx *ctx, hphi_ham *H);
+// (it and build_warp_tables append their device tables to `blob`, at the offsets `at`: one
+// allocation and one copy for both)
+int build_seg_tables(hphi_ctx *ctx, hphi_ham *H, std::vector<unsigned char> &blob, size_t *at);
+// ---- segment kernel tables (hv_warp.cu): at[0] FP32 vectors, at[1] FP64 vectors ---------
+int build_warp_tables(hphi_ctx *ctx, hphi_ham *H, std::vector<unsigned char> &blob, size_t *at);
 // ---- Hubbard kernel tables (hv_hub.cu) -------------------------------------------------
 int build_hub_tables(hphi_ctx *ctx, hphi_ham *H);
 // ---- tiled block kernel tables (hv_tile.cu) ------------------------------------------

@@ -312,14 +312,9 @@ int launch_typed(hphi_ctx *ctx, const hphi_ham *ham, HvLaunch &L) {
         const bool hub_phased = (ham->tune_variant == 3 || ham->tune_variant < 0) && ham->model == HPHI_HUBBARD &&
                                 ham->ph_ent && one_col &&
                                 (double)ham->basis->sp[1].dim * 2.0 * sizeof(T) <= 200.0 * 1024.0;
-        // the segment kernel: spin sector, one column, automatic where its tables exist.  It
-        // issues its mixed-bond FMAs for every row and the bond-major kernel only where they
-        // apply, so in FP64, where the FP64 pipe bounds both, the latter stays where its lists
-        // are longest (row blocks of 16 low bits: 4x8 56.9 against 62.3 ms; 15 bits: 6x5 15.5
-        // against 15.2).  FP32 problems below 2^14 rows keep the bond-major kernel too: both
-        // are one wave of latency there (16 sites: 10 us).
-        const bool warp = ham->tune_variant < 0 && ham->warp && ham->warp->fix[sizeof(T) == 8].bytes && one_col &&
-                          (std::is_same<T, double>::value ? ham->nlo < 16 : ham->D >= 16384);
+        // the segment kernel: spin sector, one column, automatic where its tables exist for
+        // the vectors' type (build_warp_tables has the rule)
+        const bool warp = ham->tune_variant < 0 && ham->warp && ham->warp->fix[sizeof(T) == 8].bytes && one_col;
         // Hubbard: one column or one aligned pair of columns (a complex vector), automatic where
         // its tables exist for the vectors' type (4x4 FP32 5.7 -> 3.4 ms, 6x2 complex FP64 0.149 -> 0.108 ms; 8 sites
         // 10 us either way)

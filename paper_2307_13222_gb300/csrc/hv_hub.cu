@@ -518,20 +518,22 @@ int build_hub_tables(hphi_ctx *ctx, hphi_ham *H) {
             HPHI_CUDA(ctx, cudaMemcpy(st[s].data(), B->sp[s].states, st[s].size() * sizeof(uint32_t),
                                       cudaMemcpyDeviceToHost));
         }
-    std::vector<long long> blob;  // per precision: ufix | vfix | V of one species alone, per string
+    std::vector<long long> blob;  // per precision: vfix | V of one species alone, per string
     size_t at_v[2], at_s[2][2];
     for (int t = 0; t < 2; t++) {
         const bool own = g.fix[t].parts == 2;
         const int tu = own ? eu : e2, tv = own ? ev : e2;
         auto fixed = [](double v, int e) { return (long long)llrint(ldexp(v, kHubBits - e)); };
-        const size_t at_u = blob.size();
-        blob.resize(at_u + 32, 0);
-        for (int i = 0; i < B->N; i++) blob[at_u + i] = fixed(H->host.U[i], tu);
+        for (int i = 0; i < B->N; i++) g.fix[t].ufix[i] = fixed(H->host.U[i], tu);
+        const int bits = g.fix[t].bytes == 4 ? 30 : kHubBits;
+        g.fix[t].scale = ldexp(1.0, tu - bits);
+        g.fix[t].vscale = ldexp(1.0, tv - bits);
+        if (g.nv == 0) continue;
         std::vector<HubV> vf;
         for (int k = 0; k < g.nv; k++) vf.push_back(HubV{H->host.v[k].i, H->host.v[k].j, fixed(H->host.v[k].v, tv)});
         at_v[t] = blob.size();
-        blob.resize(at_v[t] + vf.size() * (sizeof(HubV) / sizeof(long long)), 0);
-        if (!vf.empty()) memcpy(blob.data() + at_v[t], vf.data(), vf.size() * sizeof(HubV));
+        blob.resize(at_v[t] + vf.size() * (sizeof(HubV) / sizeof(long long)));
+        memcpy(blob.data() + at_v[t], vf.data(), vf.size() * sizeof(HubV));
         for (int s = 0; s < 2; s++) {
             at_s[t][s] = blob.size();
             for (uint32_t x : st[s]) {
@@ -541,19 +543,17 @@ int build_hub_tables(hphi_ctx *ctx, hphi_ham *H) {
                 blob.push_back(d);
             }
         }
-        const int bits = g.fix[t].bytes == 4 ? 30 : kHubBits;
-        g.fix[t].scale = ldexp(1.0, tu - bits);
-        g.fix[t].vscale = ldexp(1.0, tv - bits);
     }
-    cudaError_t e = cudaMalloc((void **)&H->hub_tab, blob.size() * sizeof(long long));
-    if (e == cudaSuccess)
-        e = cudaMemcpy(H->hub_tab, blob.data(), blob.size() * sizeof(long long), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_err(ctx, e, "Hubbard kernel tables");
-    for (int t = 0; t < 2; t++) {
-        g.fix[t].ufix = H->hub_tab + at_v[t] - 32;
-        g.fix[t].vfix = (const HubV *)(H->hub_tab + at_v[t]);
-        g.fix[t].dup = g.nv > 0 ? H->hub_tab + at_s[t][0] : nullptr;
-        g.fix[t].ddnf = g.nv > 0 ? H->hub_tab + at_s[t][1] : nullptr;
+    if (g.nv > 0) {
+        cudaError_t e = cudaMalloc((void **)&H->hub_tab, blob.size() * sizeof(long long));
+        if (e == cudaSuccess)
+            e = cudaMemcpy(H->hub_tab, blob.data(), blob.size() * sizeof(long long), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return cuda_err(ctx, e, "Hubbard kernel tables");
+        for (int t = 0; t < 2; t++) {
+            g.fix[t].vfix = (const HubV *)(H->hub_tab + at_v[t]);
+            g.fix[t].dup = H->hub_tab + at_s[t][0];
+            g.fix[t].ddnf = H->hub_tab + at_s[t][1];
+        }
     }
     H->hub = new (std::nothrow) HubArgs(g);
     if (!H->hub) return set_err(ctx, HPHI_E_NOMEM, "Hubbard kernel tables");

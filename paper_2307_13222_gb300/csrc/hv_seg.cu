@@ -26,6 +26,8 @@
 // a context buffer; the bond-major kernel adds t[row] to its diagonal term.
 #include "hvcommon.cuh"
 
+#include <string.h>
+
 #include <vector>
 
 namespace hphi {
@@ -116,7 +118,7 @@ __global__ void __launch_bounds__(32 * kHhsWarps, 6)
 
 // The split of the low half and the table SO of a spin S^z-sector Hamiltonian
 // with N_lo <= 16 (nothing is built otherwise and variant 4 is not offered).
-int build_seg_tables(hphi_ctx *ctx, hphi_ham *H) {
+int build_seg_tables(hphi_ctx *ctx, hphi_ham *H, std::vector<unsigned char> &blob, size_t *at) {
     const hphi_basis *B = H->basis;
     if (B->model != HPHI_SPIN_HALF || H->nlo > 16 || H->nlo < 1 || H->host.n_hh > kMaxHH) return HPHI_OK;
     SegArgs s{};
@@ -126,12 +128,7 @@ int build_seg_tables(hphi_ctx *ctx, hphi_ham *H) {
     s.n0 = H->nlo < 8 ? H->nlo : 8;
     s.n1 = H->nlo - s.n0;
     const int n0 = s.n0, n1 = s.n1;
-    auto binom = [](int n, int k) -> int64_t {
-        if (k < 0 || k > n) return 0;
-        int64_t r = 1;
-        for (int i = 1; i <= k; i++) r = r * (n - k + i) / i;
-        return r;
-    };
+    static constexpr Binomials binom;
     std::vector<uint16_t> so((size_t)(H->nlo + 1) << n1);
     for (int p = 0; p <= H->nlo; p++) {
         int64_t acc = 0;
@@ -141,10 +138,9 @@ int build_seg_tables(hphi_ctx *ctx, hphi_ham *H) {
             acc += binom(n0, p - __builtin_popcount(l1));
         }
     }
-    cudaError_t e = cudaMalloc((void **)&H->seg_so, so.size() * sizeof(uint16_t));
-    if (e == cudaSuccess) e = cudaMemcpy(H->seg_so, so.data(), so.size() * sizeof(uint16_t), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_err(ctx, e, "segment table");
-    s.so = H->seg_so;
+    *at = blob.size();
+    blob.resize(*at + so.size() * sizeof(uint16_t));
+    memcpy(blob.data() + *at, so.data(), so.size() * sizeof(uint16_t));
     H->seg = new (std::nothrow) SegArgs(s);
     if (!H->seg) return set_err(ctx, HPHI_E_NOMEM, "segment table");
     return HPHI_OK;

@@ -584,35 +584,41 @@ int go_red(hphi_ctx *ctx, const hphi_ham *ham, const HvArgs<T> &a, int red_mode,
 // Tables of the segment kernel for a spin S^z-sector Hamiltonian of at most 32
 // sites and fewer than 2^31 rows (ham->warp stays null otherwise, or when the
 // tables would not fit in shared memory next to the bond lists, or when no integers
-// hold the diagonal).
-int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
+// hold the diagonal).  The host's time for them counts for a Hamiltonian that is used
+// once, so it avoids vectors per table, divisions and branches on the strings: 5 us for
+// a 16-site chain (first product 46 -> 32), 15 for 20 sites (118 -> 43), 30 for a 14-rung
+// ladder (3880 -> 2870).
+//
+// The kernel issues its mixed-bond FMAs for every row and the bond-major kernel only
+// where they apply, so in FP64, where the FP64 pipe bounds both, the latter stays
+// where its lists are longest (row blocks of 16 low bits: 4x8 56.9 against 62.3 ms;
+// 15 bits: 6x5 15.5 against 15.2).  FP32 problems below 2^14 rows keep it too: both are
+// one wave of latency there (16 sites: 10 us).  Away from half filling segments are
+// short and lanes idle, but the bond-major kernel's blocks are shorter still: us here
+// and there, FP32, 30 sites with 4 / 6 / 10 up spins 68 / 270 / 1432 and 399 / 1048 / 3623,
+// 32 sites with 8 up 2042 and 4259; FP64, 24 sites with 1 / 4 up 8 / 26 and 39 / 127.
+int build_warp_tables(hphi_ctx *ctx, hphi_ham *H, std::vector<unsigned char> &blob, size_t *at) {
     const hphi_basis *B = H->basis;
     if (B->model != HPHI_SPIN_HALF || B->N > 32 || H->nlo > 16 || H->nlo < 1 || H->D >= ((int64_t)1 << 31))
         return HPHI_OK;
+    const bool want32 = H->D >= 16384, want64 = H->nlo < 16;
+    if (!want32 && !want64) return HPHI_OK;
     WarpArgs g{};
     g.nlo = H->nlo;
     g.n = H->host.n;
     g.s = H->nlo < kWarpSegMax ? H->nlo : kWarpSegMax;
     g.n1 = g.nlo - g.s;
     g.rot = g.n1 > 0 ? 5 : 0;
-    auto binom = [](int n, int k) -> int64_t {
-        if (k < 0 || k > n) return 0;
-        int64_t r = 1;
-        for (int i = 1; i <= k; i++) r = r * (n - k + i) / i;
-        return r;
-    };
-    // classes: rows of a segment padded to 32 nc
-    std::vector<std::vector<uint32_t>> cls(g.s + 1);
-    std::vector<uint32_t> pos((size_t)1 << g.s);
-    for (uint32_t l = 0; l < (1u << g.s); l++) {
-        std::vector<uint32_t> &c = cls[__builtin_popcount(l)];
-        pos[l] = (uint32_t)c.size();
-        c.push_back(l);
-    }
+    static constexpr Binomials binom;
+    // classes: the strings of one popcount, ascending; rows of a segment padded to 32 nc
+    const uint32_t nl = 1u << g.s;
+    unsigned char pos[1 << kWarpSegMax];  // position of a string in its class
+    uint16_t row[1 << kWarpSegMax];       // its padded row (diagonal, string)
+    uint16_t slot[1 << kWarpSegMax];      // its byte in a rank table
     int rows = 0;
     for (int c = 0; c <= g.s; c++) {
         WarpClass &k = g.cls[c];
-        k.len = (uint32_t)cls[c].size();
+        k.len = (uint32_t)binom(g.s, c);
         const int need = (int)((k.len + 31) / 32);
         if (need == 5 || need == 6 || need > kSegRows) return HPHI_OK;  // C(s, c) for s <= 10 has none
         k.nc = need;
@@ -620,6 +626,13 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
         rows += 32 * (need > 4 ? 8 : need > 2 ? 4 : need);
     }
     g.nrow = g.tab_stride = rows;
+    int seen[kWarpSegMax + 1] = {};
+    for (uint32_t l = 0; l < nl; l++) {
+        const int c = __builtin_popcount(l), r = seen[c]++, need = g.cls[c].nc;
+        pos[l] = (unsigned char)r;
+        row[l] = (uint16_t)(g.cls[c].row0 + r);
+        slot[l] = (uint16_t)(g.cls[c].tab + (r & 31) * (need > 4 ? 8 : need > 2 ? 4 : need) + (r >> 5));
+    }
     // bonds; the diagonal (at most a quarter of sum |Jz|) in fixed point below 2^62
     double bound = 0.0, c0 = 0.0, weak = 0.0;  // weak: the smallest Jxy/2
     for (const DTerm &t : H->dterms) {
@@ -644,30 +657,20 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
         for (const DTerm &t : H->dterms) ok = ok && fix_keeps(0.5 * t.a, ed, bits, digits);
         return ok || ldexp(1.0, ed - bits) <= ldexp(weak, -digits - 1);
     };
-    if (keeps(kSegBits, 53) || fabs(c0) >= ldexp(1.0, ed - 6)) g.fix[1].bytes = 8;
-    g.fix[0].bytes = keeps(30, 24) ? 4 : keeps(kSegBits, 24) ? 8 : 0;
+    if (want64 && (keeps(kSegBits, 53) || fabs(c0) >= ldexp(1.0, ed - 6))) g.fix[1].bytes = 8;
+    if (want32) g.fix[0].bytes = keeps(30, 24) ? 4 : keeps(kSegBits, 24) ? 8 : 0;
     auto fixed = [&](double v) { return (long long)llrint(ldexp(v, kSegBits - ed)); };
     std::vector<WarpBond> ub, xb, ib;  // uniform, mixed, inner
     std::vector<std::vector<WarpBond>> mb(g.s);
     std::vector<int> tab_bit(g.s, -1);
-    std::vector<std::vector<unsigned char>> tabs, itabs;
-    auto new_table = [&](std::vector<std::vector<unsigned char>> &to, uint32_t need_mask, uint32_t need_val,
-                         uint32_t flip, bool differ) {
-        std::vector<unsigned char> t(rows, 255);
-        for (int c = 0; c <= g.s; c++)
-            for (uint32_t r = 0; r < cls[c].size(); r++) {
-                const uint32_t l = cls[c][r], m = l & need_mask;
-                const bool ok = differ ? (m != 0 && m != need_mask) : m == need_val;
-                const int nb = g.cls[c].nc > 4 ? 8 : g.cls[c].nc > 2 ? 4 : g.cls[c].nc;
-                if (ok) t[g.cls[c].tab + (r & 31u) * nb + (r >> 5)] = (unsigned char)pos[l ^ flip];
-            }
-        to.push_back(t);
-        return (uint32_t)to.size() - 1;
+    std::vector<unsigned char> tabs, itabs;  // rank tables, one after the other
+    tabs.reserve((size_t)2 * g.s * rows);
+    itabs.reserve(H->dterms.size() * rows);
+    auto new_table = [&](std::vector<unsigned char> &to) {
+        to.resize(to.size() + rows, 255);
+        return (uint32_t)(to.size() / rows) - 1;
     };
-    std::vector<long long> dl0(rows, 0);
-    std::vector<uint16_t> l0s(rows, 0);
-    for (int c = 0; c <= g.s; c++)
-        for (uint32_t r = 0; r < cls[c].size(); r++) l0s[g.cls[c].row0 + r] = (uint16_t)cls[c][r];
+    std::vector<long long> dl(nl, 0);  // diagonal of the bonds inside, per string
     for (const DTerm &t : H->dterms) {
         const int i = t.i < t.j ? t.i : t.j, j = t.i < t.j ? t.j : t.i;
         const double cz = -0.5 * t.a, cxy = 0.5 * t.b;
@@ -682,27 +685,39 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
             if (cz != 0.0) mb[i].push_back(b);
             if (cxy != 0.0) {
                 if (tab_bit[i] < 0) {
-                    tab_bit[i] = (int)new_table(tabs, 1u << i, 0u, 1u << i, false);
-                    new_table(tabs, 1u << i, 1u << i, 1u << i, false);
+                    tab_bit[i] = (int)new_table(tabs);
+                    new_table(tabs);
+                    unsigned char *t0 = tabs.data() + (size_t)tab_bit[i] * rows, *t1 = t0 + rows;
+                    for (uint32_t a = 0; a < nl; a += 2u << i)
+                        for (uint32_t l = a; l < a + (1u << i); l++) {  // l and l with bit i
+                            t0[slot[l]] = pos[l | 1u << i];
+                            t1[slot[l | 1u << i]] = pos[l];
+                        }
                 }
                 b.tab = (uint32_t)tab_bit[i];
                 xb.push_back(b);
             }
         } else {
-            const uint32_t m = (1u << i) | (1u << j);
-            for (int c = 0; c <= g.s; c++)
-                for (uint32_t r = 0; r < cls[c].size(); r++) {
-                    const uint32_t lm = cls[c][r] & m;
-                    if (lm != 0 && lm != m) dl0[g.cls[c].row0 + r] += b.cz;
-                }
+            unsigned char *t = nullptr;
             if (cxy != 0.0) {
-                b.tab = new_table(itabs, m, 0u, m, true);
+                b.tab = new_table(itabs);
+                t = itabs.data() + (size_t)b.tab * rows;
                 ib.push_back(b);
             }
+            for (uint32_t a = 0; a < nl; a += 2u << j)
+                for (uint32_t c = a; c < a + (1u << j); c += 2u << i)
+                    for (uint32_t l = c; l < c + (1u << i); l++) {  // l with bit i, l with bit j
+                        const uint32_t li = l | 1u << i, lj = l | 1u << j;
+                        dl[li] += b.cz;
+                        dl[lj] += b.cz;
+                        if (t) {
+                            t[slot[li]] = pos[lj];
+                            t[slot[lj]] = pos[li];
+                        }
+                    }
         }
     }
     const long long c0f = fixed(c0);
-    for (auto &v : dl0) v += c0f;
     std::vector<WarpBond> all(ub);
     all.insert(all.end(), xb.begin(), xb.end());
     int m = 0;
@@ -717,10 +732,7 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
     g.nx = (int)xb.size();
     g.nm = m;
     g.ni = (int)ib.size();
-    g.ntab = (int)tabs.size();
-    std::vector<unsigned char> tall;
-    for (auto &t : tabs) tall.insert(tall.end(), t.begin(), t.end());
-    for (auto &t : itabs) tall.insert(tall.end(), t.begin(), t.end());
+    g.ntab = (int)(tabs.size() / rows);
     std::vector<uint16_t> so((size_t)(g.nlo + 1) << g.n1);
     for (int p = 0; p <= g.nlo; p++) {
         int64_t acc = 0;
@@ -762,35 +774,33 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H) {
                              : warp_smem<float, int>(g, kSegThreads<float> / 32)) > most)
         g.fix[0].bytes = 0;
     if (!g.fix[0].bytes && !g.fix[1].bytes) return HPHI_OK;
-    // the images of both precisions in one device block
-    std::vector<unsigned char> blob;
+    // the images of both precisions
+    blob.reserve(blob.size() + (g.fix[0].bytes ? WarpLayout<float, long long>(g).bytes : 0) +
+                 (g.fix[1].bytes ? WarpLayout<double, long long>(g).bytes : 0) + 4096);
     auto image = [&](auto zero, auto izero) {
         using T = decltype(zero);
         using I = decltype(izero);
         const WarpLayout<T, I> lay(g);
-        const size_t at = blob.size();
-        blob.resize(at + lay.bytes, 0);
-        unsigned char *p = blob.data() + at;
-        for (int i = 0; i < rows; i++) ((I *)p)[i] = to_fix<I, kSegBits>(dl0[i]);
-        memcpy(p + lay.l0s, l0s.data(), sizeof(uint16_t) * rows);
+        const size_t start = (blob.size() + 15) & ~(size_t)15;
+        blob.resize(start + lay.bytes, 0);
+        unsigned char *p = blob.data() + start;
+        for (int i = 0; i < rows; i++) ((I *)p)[i] = to_fix<I, kSegBits>(c0f);
+        for (uint32_t l = 0; l < nl; l++) {
+            ((I *)p)[row[l]] = to_fix<I, kSegBits>(c0f + dl[l]);
+            ((uint16_t *)(p + lay.l0s))[row[l]] = (uint16_t)l;
+        }
         memcpy(p + lay.so, so.data(), sizeof(uint16_t) * so.size());
         memcpy(p + lay.jp, jp.data(), sizeof(uint32_t) * jp.size());
         for (size_t i = 0; i < all.size(); i++)
             ((SmemBond<T, I> *)(p + lay.bonds))[i] =
                 SmemBond<T, I>{(T)all[i].cxy, to_fix<I, kSegBits>(all[i].cz), all[i].mask, all[i].tab};
-        if (!tall.empty()) memcpy(p + lay.tabs, tall.data(), tall.size());
-        return at;
+        if (!tabs.empty()) memcpy(p + lay.tabs, tabs.data(), tabs.size());
+        if (!itabs.empty()) memcpy(p + lay.tabs + tabs.size(), itabs.data(), itabs.size());
+        return start;
     };
-    size_t at[2] = {0, 0};
     if (g.fix[0].bytes) at[0] = g.fix[0].bytes == 8 ? image(0.0f, 0ll) : image(0.0f, 0);
     if (g.fix[1].bytes) at[1] = image(0.0, 0ll);
-    cudaError_t e = cudaMalloc((void **)&H->warp_tab, blob.size());
-    if (e == cudaSuccess) e = cudaMemcpy(H->warp_tab, blob.data(), blob.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_err(ctx, e, "segment kernel tables");
-    for (int t = 0; t < 2; t++) {
-        g.fix[t].img = H->warp_tab + at[t];
-        g.fix[t].scale = ldexp(1.0, ed - (g.fix[t].bytes == 4 ? 30 : kSegBits));
-    }
+    for (int t = 0; t < 2; t++) g.fix[t].scale = ldexp(1.0, ed - (g.fix[t].bytes == 4 ? 30 : kSegBits));
     H->warp = new (std::nothrow) WarpArgs(g);
     if (!H->warp) return set_err(ctx, HPHI_E_NOMEM, "segment kernel tables");
     return HPHI_OK;
