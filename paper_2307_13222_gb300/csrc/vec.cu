@@ -444,9 +444,11 @@ __device__ __forceinline__ Pack<T> load_pack(const T *__restrict__ p, int64_t i,
 
 // FP32 data: partials[block][j] = sum over the block's tiles of <V_j, w>.  Per
 // tile, a lane forms its partial products for J vectors at a time (8 rows
-// each); a transposing butterfly leaves in lane l the warp's sum for vector
-// j0 + l mod J, which lane l adds to the warp's FP64 slot.  The block then sums
-// its warps in order (deterministic).  Bound by HBM: 80 passes over 1 to 40
+// each); a transposing butterfly leaves in lane l a half-warp's sum, 128 rows, for
+// vector j0 + l mod J (256 rows in FP32 have 1.4 times the rounding error where the
+// products have one sign); the halves join in FP64 and lane l adds them to the
+// warp's FP64 slot.  The block then sums its warps in order (deterministic).
+// Bound by HBM: 80 passes over 1 to 40
 // vectors of 47 MB take 12.2 ms, the time of their bytes at 6.6 TB/s (20.2 ms
 // with 4-byte loads of four separate rows and groups of 32).
 template <typename T, int J, bool FULL>
@@ -482,8 +484,10 @@ __device__ __forceinline__ void mdot_group(int64_t n, int64_t ld, int j0, int nv
         }
     }
 #pragma unroll
-    for (int s2 = J; s2 < 32; s2 <<= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], s2);
-    if (lane < J && j0 + lane < nv) acc[j0 + lane] += (double)v[0];
+    for (int s2 = J; s2 < 16; s2 <<= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], s2);
+    double d = (double)v[0];  // 128 rows; the half-warps join in FP64
+    d += __shfl_xor_sync(0xffffffffu, d, 16);
+    if (lane < J && j0 + lane < nv) acc[j0 + lane] += d;
 }
 
 template <typename T, bool FULL>
