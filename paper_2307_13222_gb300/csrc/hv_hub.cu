@@ -36,6 +36,7 @@
 
 #include <algorithm>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 namespace hphi {
@@ -133,17 +134,21 @@ __global__ void __launch_bounds__(NT, MINB)
     __shared__ int nup[U];
     __shared__ I du[U];
     const HamDesc &D = *a.P.desc;
-    // alpha goes into the coefficients of one column (RED 2 needs H x itself)
-    constexpr bool FOLD = C == 1 && RED != 2;
-    T al[C], ga[C];
+    __shared__ T al_sm[C];  // (registers less through the hops)
+    T ga[C];
 #pragma unroll
-    for (int c = 0; c < C; c++) {
-        al[c] = (T)(a.alpha_dev ? a.alpha_dev[c] : a.alpha[c]);
-        ga[c] = (T)(a.gamma_dev ? a.gamma_dev[c] : a.gamma[c]);
+    for (int c = 0; c < C; c++) ga[c] = (T)(a.gamma_dev ? a.gamma_dev[c] : a.gamma[c]);
+    // FP64 hops are taken over the diagonal's scale (a power of two, so exact) and H x is
+    // scaled with alpha in one multiplication: the FP64 pipe is the bound.  FP32 ones are
+    // not: the scaled sums of vectors above 1e19 would overflow.
+    constexpr bool PRE = sizeof(T) == 8;
+    const T dscale = (T)fx.scale, vscale = (T)(PRE ? fx.vscale / fx.scale : fx.vscale);
+    const T cscale = (T)(PRE ? 1.0 / fx.scale : 1.0);
+    if (threadIdx.x < C) {
+        const T al = (T)(a.alpha_dev ? a.alpha_dev[threadIdx.x] : a.alpha[threadIdx.x]);
+        al_sm[threadIdx.x] = PRE && RED != 2 ? al * dscale : al;
     }
-    const T fold = FOLD ? al[0] : (T)1;
-    const T dscale = (T)fx.scale * fold, vscale = (T)fx.vscale * fold;
-    for (int i = threadIdx.x; i < D.n_ncoef; i += NT) coef[i] = (T)D.coef[i] * fold;
+    for (int i = threadIdx.x; i < D.n_ncoef; i += NT) coef[i] = (T)D.coef[i] * cscale;
     const T be = (T)a.beta;
     const bool use_beta = a.beta != 0.0, use_v = a.v != nullptr;
     const T *__restrict__ X = a.x;
@@ -163,7 +168,7 @@ __global__ void __launch_bounds__(NT, MINB)
             hp.c = (T)0;
             if (h < g.nh && e < a.P.up_cnt[h]) {
                 hp.row = a.P.up_tgt[(int64_t)e * g.nh + h] * ddn;
-                hp.c = (T)D.coef[a.P.up_cf[(int64_t)e * g.nh + h]] * fold;
+                hp.c = coef[a.P.up_cf[(int64_t)e * g.nh + h]];
             }
             hops[i] = hp;
         }
@@ -235,27 +240,27 @@ __global__ void __launch_bounds__(NT, MINB)
                 I d[U];
 #pragma unroll
                 for (int u = 0; u < U; u++) d[u] = dl + du[u];
-                T dv[U];  // the V part, where it is summed apart
-                if constexpr (sizeof(T) == 8) {
+                T dt[U];
+                if (parts == 2) {  // the V part apart (FP64)
+                    T dv[U];
+                    add(tab + U * g.ngrp * 64, d);
 #pragma unroll
-                    for (int u = 0; u < U; u++) dv[u] = (T)0;
-                    if (parts == 2) {
-                        add(tab + U * g.ngrp * 64, d);
-#pragma unroll
-                        for (int u = 0; u < U; u++) {
-                            dv[u] = (T)d[u] * vscale;
-                            d[u] = 0;
-                        }
+                    for (int u = 0; u < U; u++) {
+                        dv[u] = (T)d[u] * vscale;
+                        d[u] = 0;
                     }
+                    add(tab, d);
+#pragma unroll
+                    for (int u = 0; u < U; u++) dt[u] = (T)d[u] + dv[u];
+                } else {
+                    add(tab, d);
+#pragma unroll
+                    for (int u = 0; u < U; u++) dt[u] = PRE ? (T)d[u] : (T)d[u] * dscale;
                 }
-                add(tab, d);
 #pragma unroll
                 for (int u = 0; u < U; u++) {
-                    T dt;
-                    if constexpr (sizeof(T) == 8) dt = fma((T)d[u], dscale, dv[u]);
-                    else dt = (T)d[u] * dscale;
 #pragma unroll
-                    for (int c = 0; c < C; c++) acc[b][u * C + c] = dt * x.e[u * C + c];
+                    for (int c = 0; c < C; c++) acc[b][u * C + c] = dt[u] * x.e[u * C + c];
                 }
             }
             // the down hops wait on shared memory, the up hops on L2: odd warps take them the
@@ -317,17 +322,23 @@ __global__ void __launch_bounds__(NT, MINB)
                 }
             }
             // epilogue: y = alpha (H x) + beta y + gamma v, old values loaded before any store
-#pragma unroll
-            for (int b = 0; b < QB; b++) {
-                if (!on[b]) continue;
+            auto finish = [&](int b, auto times_alpha) {
                 const HubPack<T> x = xs[q[b]];
                 T out[P];
+                if constexpr (PRE && RED == 2) {
+#pragma unroll
+                    for (int i = 0; i < P; i++) acc[b][i] *= dscale;
+                }
+                T al[C];
+#pragma unroll
+                for (int c = 0; c < C; c++) al[c] = al_sm[c];
 #pragma unroll
                 for (int u = 0; u < U; u++)
 #pragma unroll
                     for (int c = 0; c < C; c++) {
                         const T hx = acc[b][u * C + c], other = acc[b][u * C + (C == 2 ? c ^ 1 : c)];
-                        out[u * C + c] = FOLD ? hx : al[c] * (C == 2 && a.swap ? other : hx);
+                        if constexpr (decltype(times_alpha)::value) out[u * C + c] = al[c] * (C == 2 && a.swap ? other : hx);
+                        else out[u * C + c] = hx;
                     }
                 if (use_beta) {
 #pragma unroll
@@ -368,6 +379,15 @@ __global__ void __launch_bounds__(NT, MINB)
                         if constexpr (RED == 3) racc[0][c].add(o[c], o[c]);
                     }
                 }
+            };
+            // one FP32 column with alpha = 1 (the usual product) has an epilogue of its own: the
+            // multiplications cost it 2 to 9 % at 12 to 14 sites
+            const bool plain = C == 1 && !PRE && al_sm[0] == (T)1;
+#pragma unroll
+            for (int b = 0; b < QB; b++) {
+                if (!on[b]) continue;
+                if (plain) finish(b, std::false_type());
+                else finish(b, std::true_type());
             }
         }
     }

@@ -64,6 +64,15 @@ constexpr int kSegStage = 256;  // staged values per warp (a slot behind every s
 constexpr int kSegBits = 62;  // the diagonal lies below 2^62 grid steps
 constexpr int kSegRows = 8;   // rows of a lane held in registers (C(10, 5) = 252 rows per segment)
 
+// FP64 couplings are stored over the diagonal's scale (a power of two, so exact) and H x
+// is scaled with alpha in one multiplication: the FP64 pipe is the bound.  FP32 ones are
+// not: the scaled sums of vectors above 1e19 would overflow.  There alpha goes into the
+// couplings and the diagonal's scale (RED 2 needs H x itself): a multiplication per row
+// costs 20 Lanczos steps of the 6x5 lattice 3 %, and their alphas are no closer to 64
+// bits with it (6x4 lattice, 8 start vectors: 1.36e-7 with, 1.33e-7 without).
+template <typename T> constexpr bool seg_scaled = sizeof(T) == 8;
+template <typename T, int RED> constexpr bool seg_fold = !seg_scaled<T> && RED != 2;
+
 // A bond of the image, in T's precision.
 struct WarpBond {     // a bond as the builder collects it
     double cxy;       // Jxy/2
@@ -163,6 +172,10 @@ struct WarpLayout {
     }
 };
 
+__device__ __forceinline__ double seg_diag(long long d, double) { return (double)d; }
+template <typename I>
+__device__ __forceinline__ float seg_diag(I d, float scale) { return (float)d * scale; }
+
 // What a warp needs to know of its segment.
 template <typename T, typename I>
 struct Seg {
@@ -181,28 +194,34 @@ struct Seg {
 };
 template <typename T>
 struct Epi {
-    T al, ga, be, dscale;
+    const T *al;  // in shared memory: one register less through the bonds
+    T ga, be, dscale;
     bool use_beta, use_v;
     uint64_t keep, stream;
 };
 
 // Epilogue of NC rows row, row + 32, ... (the last one only if `tail`; xs: their
 // x, 32 apart): the old y and v of all rows are loaded before the first store.
-// acc is H x, times alpha unless RED is 2.
+// acc is H x, in FP64 over the diagonal's scale, in FP32 times alpha unless RED is 2.
 template <typename T, int NC, int RED>
 __device__ __forceinline__ void seg_out(const HvArgs<T> &a, const Epi<T> &e, uint32_t row, bool tail, const T *xs,
                                         T (&acc)[NC], RedAcc<T> (&racc)[RED == 2 ? 3 : 1]) {
     if constexpr (RED == 2) {
 #pragma unroll
         for (int c = 0; c < NC; c++) {
+            if constexpr (seg_scaled<T>) acc[c] = e.dscale * acc[c];
             if (c + 1 < NC || tail) {
                 const T xo = xs[32 * c];
                 racc[0].add(xo, acc[c]);
                 racc[1].add(acc[c], acc[c]);
                 racc[2].add(xo, xo);
             }
-            acc[c] = e.al * acc[c];
         }
+    }
+    if constexpr (!seg_fold<T, RED>) {
+        const T al = *e.al;
+#pragma unroll
+        for (int c = 0; c < NC; c++) acc[c] = al * acc[c];
     }
     if (e.use_beta) {
         T t[NC];
@@ -252,7 +271,7 @@ __device__ __forceinline__ void seg_rows(const HvArgs<T> &a, const Seg<T, I> &g,
             const uint32_t l0 = g.l0s[lane + 32 * c];
             const I d = g.du + g.dl0[lane + 32 * c] + __shfl_sync(0xffffffffu, g.tlo, l0 & 31u) +
                         __shfl_sync(0xffffffffu, g.thi, l0 >> 5);
-            acc[c] = ((T)d * e.dscale) * xo[c];
+            acc[c] = seg_diag(d, e.dscale) * xo[c];
         }
     }
     __syncwarp();
@@ -336,7 +355,7 @@ __device__ __noinline__ void seg_edge(const HvArgs<T> &a, const Seg<T, I> &g, co
         const I d = g.du + g.dl0[r] + __shfl_sync(0xffffffffu, g.tlo, l0 & 31u) +
                     __shfl_sync(0xffffffffu, g.thi, l0 >> 5);
         const T xo = in ? xs[r] : (T)0;
-        T acc = ((T)d * e.dscale) * xo;
+        T acc = seg_diag(d, e.dscale) * xo;
         for (int k = 0; k < g.nib; k++) {
             const uint32_t t = g.itabs[k * g.stride + lane * nb + c];
             if (in && t != 255u) acc = fma(g.ib[k].cxy, xs[t], acc);
@@ -355,6 +374,7 @@ __global__ void __launch_bounds__(NT, MINB)
     k_hvw(const __grid_constant__ HvArgs<T> a, const __grid_constant__ WarpArgs g) {
     constexpr int W = NT / 32;
     extern __shared__ __align__(16) unsigned char s_raw[];
+    __shared__ T al_sm;
     // shared layout: per warp the bond list and the staged segment, then the
     // Hamiltonian's tables (one copy of the image in memory), then the traversal
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -376,20 +396,24 @@ __global__ void __launch_bounds__(NT, MINB)
         if (a.P.use_perm)
             for (int i = threadIdx.x; i < 512; i += NT) perm[i] = (uint16_t)block_of(a.P, i < 256 ? i : (i - 256) << 8);
         for (int i = threadIdx.x; i < W * kSegStage; i += NT) stages[i] = (T)0;
+        if (threadIdx.x == 0) {
+            al_sm = (T)(a.alpha_dev ? a.alpha_dev[0] : a.alpha[0]);
+            if constexpr (seg_scaled<T> && RED != 2) al_sm *= (T)g.fix[1].scale;
+        }
     }
     __syncthreads();
-    const T al = (T)(a.alpha_dev ? a.alpha_dev[0] : a.alpha[0]);
-    if constexpr (RED != 2) {  // alpha goes into the coefficients (RED 2 needs H x itself)
+    if constexpr (seg_fold<T, RED>) {
+        const T al = al_sm;
         for (int i = threadIdx.x; i < nlist + g.nm + g.ni; i += NT) ((SmemBond<T, I> *)ub)[i].cxy *= al;
         __syncthreads();
     }
     Epi<T> e;
     e.keep = spol(a.P.hints, 0);
     e.stream = spol(a.P.hints, 1);
-    e.al = al;
+    e.al = &al_sm;
     e.ga = (T)(a.gamma_dev ? a.gamma_dev[0] : a.gamma[0]);
     e.be = (T)a.beta;
-    e.dscale = (T)g.fix[sizeof(T) == 8].scale * (RED != 2 ? al : (T)1);
+    e.dscale = (T)g.fix[sizeof(T) == 8].scale * (seg_fold<T, RED> ? al_sm : (T)1);
     e.use_beta = a.beta != 0.0;
     e.use_v = a.v != nullptr;
     Seg<T, I> sg;
@@ -793,7 +817,7 @@ int build_warp_tables(hphi_ctx *ctx, hphi_ham *H, std::vector<unsigned char> &bl
         memcpy(p + lay.jp, jp.data(), sizeof(uint32_t) * jp.size());
         for (size_t i = 0; i < all.size(); i++)
             ((SmemBond<T, I> *)(p + lay.bonds))[i] =
-                SmemBond<T, I>{(T)all[i].cxy, to_fix<I, kSegBits>(all[i].cz), all[i].mask, all[i].tab};
+                SmemBond<T, I>{(T)(seg_scaled<T> ? ldexp(all[i].cxy, kSegBits - ed) : all[i].cxy), to_fix<I, kSegBits>(all[i].cz), all[i].mask, all[i].tab};
         if (!tabs.empty()) memcpy(p + lay.tabs, tabs.data(), tabs.size());
         if (!itabs.empty()) memcpy(p + lay.tabs + tabs.size(), itabs.data(), itabs.size());
         return start;

@@ -146,3 +146,23 @@ def test_few_up_strings(N, nu, nd, threads, dtype):
         hphi.hphi_apply_H(h, Vg, y)
         assert rel_err(y.double().cpu().numpy(), m.apply(x)) < tol
     assert f",{threads},I" in h.ctx.last_kernel() and h.ctx.last_kernel().startswith("k_hub<")
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32, torch.complex128, torch.complex64])
+def test_alpha_is_applied_once(dtype):
+    """y = alpha (H x) rounds H x by alpha once: bit for bit alpha times the product with
+    alpha = 1 (couplings that carry alpha would be rounded once more each).  Segment kernel
+    in FP64 too."""
+    hams = [pair("HUBBARD", 8, 4, 3, hubbard_terms(8, chain(8), t=0.7, U=3.3, V=0.3))]
+    if dtype == torch.float64:
+        hams.append(pair("SPIN_HALF", 14, 7, 0, [("XXZ", i, j, 0, 0.7, 1.1) for i, j in square(7, 2)]))
+    for m, b, h in hams:
+        x = torch.from_numpy(random_vectors(m.dim, 1, 9, complex_=dtype.is_complex, normalize=False)[:, 0].copy())
+        xd = x.to(dtype).cuda()
+        y1, ya = torch.empty_like(xd), torch.empty_like(xd)
+        hphi.hphi_apply_H(h, xd, y1)
+        for alpha in (0.8, -1.1, 0.123456789):
+            hphi.hphi_apply_H(h, xd, ya, alpha)
+            r = (lambda t: torch.view_as_real(t)) if dtype.is_complex else (lambda t: t)
+            al = torch.tensor(alpha, dtype=r(y1).dtype, device="cuda")
+            assert torch.equal(r(ya), al * r(y1)), (h.ctx.last_kernel(), alpha)
