@@ -792,7 +792,6 @@ int launch_tile(hphi_ctx *ctx, const hphi_ham *ham, HvArgs<T> &a, int red_mode, 
     const T *diag = (const T *)ham->tile_diag[prec];
     TileArgs tp = ta;
     if (ta.nout[0] >= 2 || ta.nout[1] >= 2) {
-        if (!ctx->ticket) HPHI_CUDA(ctx, cudaMalloc(&ctx->ticket, 2 * sizeof(unsigned)));
         HPHI_CUDA(ctx, cudaMemsetAsync(ctx->ticket, 0, 2 * sizeof(unsigned), ctx->stream));
         for (int p = 0; p < 2; p++) tp.ticket[p] = ta.nout[p] >= 2 ? ctx->ticket + p : nullptr;
     }
