@@ -55,12 +55,15 @@ extern "C" int hphi_ham_autotune(hphi_ctx *ctx, hphi_ham *ham, int dtype, int nv
     // candidate settings: variant x split x hints (x coop for 32-column rows, x form of the staged kernel)
     std::vector<std::vector<int>> cand;
     const bool spin = ham->model != HPHI_HUBBARD;
-    const std::vector<int> variants = spin ? std::vector<int>{-1, 0, 1, 2, 3, 4, 5} : std::vector<int>{-1, 0};
+    const std::vector<int> variants = spin ? std::vector<int>{-1, 0, 1, 2, 3, 4, 5} : std::vector<int>{-1, 0, 3};
+    // the Hubbard kernel (the automatic choice of one column or one pair) ignores the others
+    const bool hub = !spin && nr <= 2 && ham->hub && ham->hub->fix[real_of(dtype) == HPHI_F64].bytes;
     for (int v : variants)
         for (int sp : {1, 2, 4})
             for (int hi : {0, 1}) {
                 // the segment kernel (the automatic choice of one sector column): one launch form
                 if (v == -1 && spin && (sp != 1 || nr != 1 || ham->model != HPHI_SPIN_HALF)) continue;
+                if (v == -1 && hub && (sp != 1 || hi != 1)) continue;
                 // the staged kernels own a row block per thread block and take one column
                 if (v >= 2 && v <= 4 && (sp != 1 || nr != 1)) continue;
                 // the tiled kernel: 32-column rows of the full space, one launch form

@@ -166,3 +166,11 @@ def test_alpha_is_applied_once(dtype):
             r = (lambda t: torch.view_as_real(t)) if dtype.is_complex else (lambda t: t)
             al = torch.tensor(alpha, dtype=r(y1).dtype, device="cuda")
             assert torch.equal(r(ya), al * r(y1)), (h.ctx.last_kernel(), alpha)
+
+
+def test_autotune_tries_every_kernel_once():
+    """One Hubbard column: the automatic kernel in its one form, the row kernel in 6 (split x
+    hints), the bond-major kernel in 2 (hints)."""
+    m, b, h = pair("HUBBARD", 8, 4, 3, hubbard_terms(8, chain(8), t=1.0, U=4.0))
+    assert h.autotune(torch.float32, 1, reps=1)[1] == 9
+    assert h.autotune(torch.complex64, 1, reps=1)[1] == 7  # (the bond-major kernel takes one column)
