@@ -174,3 +174,28 @@ def test_autotune_tries_every_kernel_once():
     m, b, h = pair("HUBBARD", 8, 4, 3, hubbard_terms(8, chain(8), t=1.0, U=4.0))
     assert h.autotune(torch.float32, 1, reps=1)[1] == 9
     assert h.autotune(torch.complex64, 1, reps=1)[1] == 7  # (the bond-major kernel takes one column)
+
+
+# What the automatic choice is around the limits of shared memory: 12,870 down strings of 16 bytes
+# fit (k_hub), 19,448 do not, 24,310 of the FP32 bond-major kernel's 8 bytes do, 43,758 do not.
+@pytest.mark.parametrize("N,nd,f32,f64", [(16, 8, "k_hub<", "k_hub<"), (17, 7, "k_hvp<", "k_hv<"),
+                                          (17, 8, "k_hvp<", "k_hv<"), (18, 8, "k_hv<", "k_hv<")])
+def test_automatic_kernel_by_down_strings(N, nd, f32, f64):
+    m, b, h = pair("HUBBARD", N, 1, nd, hubbard_terms(N, chain(N), t=1.0, U=4.0))
+    x = random_vectors(m.dim, 1, 3, normalize=False)[:, 0]
+    for dtype, name in ((torch.float32, f32), (torch.float64, f64)):
+        xt = torch.from_numpy(x).to(dtype)
+        y = torch.empty(m.dim, dtype=dtype, device="cuda")
+        hphi.hphi_apply_H(h, xt.cuda(), y, 0.9)
+        assert h.ctx.last_kernel().startswith(name)
+        assert rel_err(y.cpu().double().numpy(), m.apply(xt.double().numpy(), 0.9)) < TOL[dtype]
+
+
+def test_bond_major_kernel_4x4_sampled():
+    """165,636,900 rows through the bond-major kernel (on request there), FP32."""
+    from test_gpu_hv import _sampled_rows
+    m, b, h = pair("HUBBARD", 16, 8, 8, hubbard_terms(16, square(4, 4), t=1.0, U=8.0))
+    h.set_tuning(variant=3)
+    rows = np.concatenate([[0, m.dim - 1], np.random.default_rng(9).integers(0, m.dim, 300)])
+    assert _sampled_rows(m, h, torch.float32, 1, rows, 44) < 1e-6
+    assert h.ctx.last_kernel().startswith("k_hvp<f32")

@@ -116,3 +116,21 @@ def test_coupling_that_is_not_finite_stays_on_its_rows(model, ncol, dtype):
     y = torch.empty_like(x)
     hphi.hphi_apply_H(h, x, y)
     assert (np.isfinite(y.cpu().numpy()) == (((s ^ (s >> 1)) & 1) == 0)[:, None]).all()
+
+
+# FP32 (above 2^14 rows, below which the bond-major kernel takes the call) at both ends of the
+# popcounts: segments of 0 to 4 and of 6 to 10 up spins, of one row to 210, most of them short.
+@pytest.mark.parametrize("N,nup", [(27, 4), (27, 23), (31, 4), (20, 7)])
+def test_segment_kernel_f32_sparse_sectors(N, nup):
+    m, b, h = pair("SPIN_HALF", N, nup, 0, _terms(N, N * 41 + nup)[:64])
+    x = torch.from_numpy(random_vectors(m.dim, 1, N, normalize=False)[:, 0]).float()
+    y = torch.from_numpy(random_vectors(m.dim, 1, N + 1, normalize=False)[:, 0]).float()
+    for alpha, beta in ((0.8, 0.0), (-1.1, 0.35)):
+        pad = torch.full((m.dim + 130,), float("nan"), device="cuda")
+        xd = pad.clone()[65:65 + m.dim].copy_(x)
+        yd = pad[65:65 + m.dim].copy_(y)
+        hphi.hphi_apply_H(h, xd, yd, alpha, beta)
+        assert h.ctx.last_kernel().startswith("k_hvw<f32")
+        want = m.apply(x.double().numpy(), alpha, beta, y.double().numpy().copy())
+        assert rel_err(yd.cpu().double().numpy(), want) < TOL[torch.float32]
+        assert pad[:65].isnan().all() and pad[65 + m.dim:].isnan().all()

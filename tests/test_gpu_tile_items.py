@@ -60,3 +60,31 @@ def test_steps(N, dtype):
         assert np.allclose(e[:2], eo, rtol=tol, atol=tol) and np.allclose(h2[:2], h2o, rtol=tol)
         assert np.allclose(logd[:2], np.log(do), atol=tol)
     assert rel_err(Vg[:, :2].cpu().numpy(), Vo / np.linalg.norm(Vo, axis=0) * np.sqrt(norm2[:2])) < tol
+
+
+@pytest.mark.parametrize("dtype", [torch.complex128, torch.complex64])
+def test_steps_over_many_tiles_repeat_bitwise(dtype):
+    """Several tiles per pass: tickets in the first pass, paced thread blocks in the second
+    (its sums in a fixed order), so a repeated step gives the same bits."""
+    N = 20
+    m, b, h = pair("SPIN_HALF_GC", N, 0, 0, _terms(N, N, chain(N)))
+    tol = 1e-11 if dtype == torch.complex128 else 2e-5
+    V0 = random_vectors(m.dim, 16, 7, complex_=True)
+    runs = []
+    for _ in range(2):
+        V = torch.from_numpy(V0).to(dtype).cuda().contiguous()
+        ev = hphi.hphi_time_step(h, V, 0.02, 3)
+        norm2 = np.zeros(16)
+        tp = hphi.hphi_tpq_step(h, V, 0.05, 2, norm2)
+        assert h.ctx.last_kernel().startswith("k_tile<")
+        runs.append((V, [np.asarray(a) for a in (*ev, *tp, norm2)]))
+    assert torch.equal(torch.view_as_real(runs[0][0]), torch.view_as_real(runs[1][0]))
+    assert all(np.array_equal(a, c) for a, c in zip(runs[0][1], runs[1][1]))
+    Vo = V0[:, :1].copy()
+    no, eo, noo = m.time_step(Vo, 0.02, 3)
+    n2, e = runs[0][1][:2]
+    assert np.allclose(n2[:1], no, rtol=tol) and np.allclose(e[:1], eo, rtol=tol, atol=tol)
+    eo, h2o, do = m.tpq_step(Vo, 0.05, 2)
+    e, h2, logd, norm2 = runs[0][1][4:]
+    assert np.allclose(e[:1], eo, rtol=tol, atol=tol) and np.allclose(h2[:1], h2o, rtol=tol)
+    assert rel_err(runs[0][0][:, :1].cpu().numpy(), Vo / np.linalg.norm(Vo, axis=0) * np.sqrt(norm2[:1])) < tol
