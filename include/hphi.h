@@ -165,9 +165,15 @@ HPHI_API int64_t hphi_ham_dim(const hphi_ham *ham);
  *   HPHI_TUNE_SPLIT       thread blocks that share one row block (1..8),
  *                         fewer row blocks in flight for the same occupancy
  *   HPHI_TUNE_L2_HINTS    1 = L2 eviction-priority hints on gathers/streams
- *   HPHI_TUNE_VARIANT     -1 = automatic (default; one column of an S^z sector
- *                         takes the segment kernel, which has no number of
- *                         its own); spin models: 1 = neighbour
+ *   HPHI_TUNE_VARIANT     -1 = automatic (default).  Two kernels are taken there
+ *                         only: the segment kernel for one column of an S^z
+ *                         sector of up to 32 sites and 2^31 rows (FP64 with up
+ *                         to 30 sites, FP32 from 2^14 rows), the Hubbard kernel
+ *                         for one column or one 16-byte-packed pair (a complex
+ *                         vector) where the rows of an up string fit in shared
+ *                         memory (about 13,900 down strings); both only where
+ *                         a fixed-point diagonal keeps every coupling's digits.
+ *                         Spin models: 1 = neighbour
  *                         ranks computed on the fly from Lin's ja table, 0 =
  *                         precomputed neighbour lists (also enables the
  *                         one-thread-per-row kernel for Hubbard), 2 = staged:
