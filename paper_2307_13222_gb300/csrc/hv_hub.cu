@@ -18,13 +18,14 @@
 // else 64; FP64 vectors one grid or two, one for U and one for V, and the kernel
 // only where these cost less than the hops round.
 //
-// What bounds it: FP64 the FP64 pipe (88 % busy; a warp's down hops run as many
-// rounds as its longest list), FP32 the latency of the up-hop loads and the bank
-// conflicts of the 16-byte gathers.  ms per product, before and now: 4x4 FP32
-// 5.67 -> 3.4, FP64 17.0 -> 12.7; 7x2 ladder FP32 0.403 -> 0.148, complex FP64 1.75
-// -> 1.40; 6x2 complex FP64 0.149 -> 0.108.  (Before: the bond-major kernel,
+// What bounds it: FP64 the FP64 pipe (89 % busy; a warp's down hops run as many
+// rounds as its longest list), FP32 the latency of the up-hop loads (4x4: 6 stalls per
+// issue at 32 warps per SM, 17.9 GB from L2 at 5.4 TB/s) and the bank conflicts of the
+// 16-byte gathers (36 % of the shared-load wavefronts).  ms per product, before and
+// now: 4x4 FP32 5.66 -> 3.3, FP64 17.1 -> 12.6; 7x2 ladder FP32 0.400 -> 0.148, complex
+// FP64 1.75 -> 1.36; 6x2 complex FP64 0.149 -> 0.107.  (Before: the bond-major kernel,
 // hv_phased.cu, which walks a list per (hop pair, sign) through a shared
-// accumulator, 22 warp instructions per row against 9.5 here; for pairs the
+// accumulator, 22 warp instructions per row against 11 here; for pairs the
 // generic kernel, which issues its FMAs for every slot of a batch of eight.)
 // Tried: 8 down hops in flight 44: 3.67, 16 up hops 3.69, 512 threads 4.2, thread
 // counts that leave no lane idle 7x2 FP32 0.179.

@@ -40,12 +40,13 @@
 // and, for 16 (8) rows, 4 (8) loads per lane and their FMAs; only bonds with a site
 // inside test anything per row.  Every row sums its terms in a fixed order: deterministic.
 //
-// What bounds it: FP32 L2-to-SM traffic (about 11 reads of 128 bytes per row and
-// pass, 9 to 10 TB/s), FP64 the FP64 pipe.  Before, 8 lanes walked the bonds row
+// What bounds it: FP32 L2-to-SM traffic (22 sites, pass 1: 8.4 reads of 128 bytes
+// per row at 10.1 TB/s; 26 sites about 11 per row and pass), FP64 the FP64 pipe
+// (21-site chain, pass 1: 94 % busy, 5.5 operations per element).  Before, 8 lanes walked the bonds row
 // by row, testing each bond on each row (74 to 80 warp instructions per row and
 // pass).  ms per cTPQ step (6 stages), before and now: 26 sites of a 3-regular
-// graph FP32 118.6 -> 103, 25-site chain FP32 50.7 -> 43.4, 21-site ladder FP64
-// 25.5 -> 14.2, 22 sites FP64 57 -> 29.5.  Tried (26 sites): 24 warps per SM 123, 32
+// graph FP32 116 -> 102, 25-site chain FP32 50.7 -> 43.4, 21-site ladder FP64
+// 25.6 -> 14.2, 22 sites FP64 57 -> 29.5.  Tried (26 sites): 24 warps per SM 123, 32
 // 206 (more rows in flight leave L2 early), 2 rows per lane 122 to 217.
 #include "fixed.cuh"
 #include "hvcommon.cuh"

@@ -34,12 +34,12 @@
 // the work split is static: deterministic.  (Sec. 3.1.1: the exchange terms on
 // the bit-encoded basis.)
 //
-// What bounds it: FP32 the latency of the gathers (6x5 lattice: 13 warp
-// instructions per row, 54 % of the issue slots, DRAM 2.4 TB/s), FP64 the FP64
-// pipe (92 % busy).  Measured against the bond-major kernel (hv_phased.cu, 25
-// warp instructions per row), ms per product: 4x8 FP32 24.6 -> 14.4, 6x5 FP32
-// 6.02 -> 2.83, 14-rung ladder FP32 1.58 -> 0.52, FP64 3.83 -> 3.03, 24-site
-// chain FP64 0.39 -> 0.14, 16-site chain FP64 0.025 -> 0.010.  Splits tried: 9
+// What bounds it: FP32 the latency of the gathers (6x5 lattice: 12.8 warp
+// instructions per row, 57 % of the issue slots, DRAM 2.6 TB/s), FP64 the FP64
+// pipe (94 % busy).  Measured against the bond-major kernel (hv_phased.cu, 25
+// warp instructions per row), ms per product: 4x8 FP32 24.6 -> 14.2, 6x5 FP32
+// 6.02 -> 2.75, 14-rung ladder FP32 1.58 -> 0.49, FP64 3.92 -> 2.91, 24-site
+// chain FP64 0.39 -> 0.125, 16-site chain FP64 0.025 -> 0.010.  Splits tried: 9
 // segment bits 6x5 3.66, 8 bits 5.68 (lanes idle in short segments); 8 uniform
 // loads in flight per lane 3.27, 16: 2.87, 24: 2.79; 16 mixed loads 3.32; two
 // batches in flight at a time 5.9 (spills at 64 registers); 16 warps per SM 3.4.

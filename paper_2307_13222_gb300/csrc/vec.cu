@@ -527,8 +527,9 @@ __global__ void __launch_bounds__(kMT, 4) k_mdot_tiled(int64_t n, int64_t ld, in
 // w[r] -= sum_j c[j] V[j][r], the sum in T in order of j; with `norm`, also the
 // block's partial sum of the new w[r]^2 (partials[block]): the second projection
 // of a step leaves |w|^2 behind, without another pass over w.  Bound by HBM (81
-// passes over 1 to 40 vectors of 47 MB: 12.3 ms, 14.7 with 4-byte loads; two
-// vectors per iteration: 4 13.8, 8 13.0).
+// passes over 1 to 40 vectors of 47 MB: 12.3 ms, 7.05 TB/s of what they read and
+// write, above the copy rate, as part of w is still in L2; 14.7 ms with 4-byte
+// loads; two vectors per iteration: 4 13.8, 8 13.0).
 template <typename T, bool FULL>
 __device__ __forceinline__ void maxpy_tile(int64_t n, int64_t ld, int nv, const T *__restrict__ V, const T *cs, T *w,
                                            int64_t r0, int norm, Acc<T> &nn) {
