@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(NT, MINB)
     for (int c = 0; c < C; c++) ga[c] = (T)(a.gamma_dev ? a.gamma_dev[c] : a.gamma[c]);
     // FP64 hops are taken over the diagonal's scale (a power of two, so exact) and H x is
     // scaled with alpha in one multiplication: the FP64 pipe is the bound.  FP32 ones are
-    // not: the scaled sums of vectors above 1e19 would overflow.
+    // not: the scaled sums of vectors above 1e19 would overflow (FP64's only above 1e288).
     constexpr bool PRE = sizeof(T) == 8;
     const T dscale = (T)fx.scale, vscale = (T)(PRE ? fx.vscale / fx.scale : fx.vscale);
     const T cscale = (T)(PRE ? 1.0 / fx.scale : 1.0);
@@ -500,6 +500,8 @@ int build_hub_tables(hphi_ctx *ctx, hphi_ham *H) {
     for (int k = 0; k < g.nv; k++) vbound += 4.0 * fabs(H->host.v[k].v);
     for (int k = 0; k < H->host.n_ncoef; k++) hop = k ? std::min(hop, fabs(H->host.coef[k])) : fabs(H->host.coef[k]);
     if (!isfinite(ubound + vbound)) return HPHI_OK;
+    for (int k = 0; k < H->host.n_ncoef; k++)
+        if (!(fabs(H->host.coef[k]) < 1e30)) return HPHI_OK;  // FP64 hops are scaled by up to 2^122
     auto grid = [](double b) {
         int e2 = 0;
         frexp(b > 0.0 ? b : 1.0, &e2);

@@ -199,3 +199,14 @@ def test_bond_major_kernel_4x4_sampled():
     rows = np.concatenate([[0, m.dim - 1], np.random.default_rng(9).integers(0, m.dim, 300)])
     assert _sampled_rows(m, h, torch.float32, 1, rows, 44) < 1e-6
     assert h.ctx.last_kernel().startswith("k_hvp<f32")
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.complex128])
+def test_huge_hop_stays_finite(dtype):
+    """Hops near the end of FP64's range (the kernel scales its couplings: not taken there)."""
+    m, b, h = pair("HUBBARD", 6, 3, 2, hubbard_terms(6, chain(6), t=1e295, U=4.0))
+    x = torch.from_numpy(random_vectors(m.dim, 1, 4, complex_=dtype.is_complex)[:, 0].copy())
+    y = torch.empty(m.dim, dtype=dtype, device="cuda")
+    hphi.hphi_apply_H(h, x.to(dtype).cuda(), y)
+    want = _h(m, x.numpy()) if dtype.is_complex else m.apply(x.numpy())
+    assert rel_err(y.cpu().numpy() / 1e295, want / 1e295) < TOL[dtype]
